@@ -26,6 +26,7 @@ namespace leg {
 namespace {
 
 constexpr int kDB = 1024;                  // Gaussians per classification block
+constexpr int kSB = 512;                   // Gaussians per scatter block
 
 struct DensifyThresholds {
     float grad_thresh, log_big, logit_min, ln16, max_screen, log_world;
@@ -34,11 +35,6 @@ struct DensifyThresholds {
 struct Fields {
     float* f[7];
 };
-
-__host__ __device__ constexpr int field_w(int f, int nc)
-{
-    return f == 4 ? 3 * nc : (f == 2 ? 4 : (f == 5 ? 8 : (f <= 1 ? 3 : 1)));
-}
 
 __global__ void densify_stats_kernel(int n, const float4* __restrict__ grad2d, const int* __restrict__ radius,
                                      float* __restrict__ acc, int* __restrict__ cnt, int* __restrict__ max_radius)
@@ -154,7 +150,7 @@ __global__ void __launch_bounds__(1024) densify_scan_kernel(unsigned* bcount, in
 }
 
 struct ScatterArgs {
-    int n, nc;
+    int n, nb;                      // Gaussians, classification blocks
     Fields p, m, v;                 // inputs
     Fields po, mo, vo;              // outputs
     const uint8_t* kind;
@@ -162,114 +158,168 @@ struct ScatterArgs {
     const unsigned long long* totals;
     const float* noise;             // [n][2][3]
     float ln16;
+    unsigned vec;                   // bit f: the six arrays of field f are 16-byte aligned
 };
 
-// Copies Gaussian src to output slot dst in every field (moments or zeros);
-// 16-byte accesses for the fields whose rows are whole multiples of 16 bytes
-// (quaternions, SH, features) when the arrays allow it, scalar ones otherwise.
-__device__ __forceinline__ void copy_gaussian(const ScatterArgs& a, size_t src, size_t dst, bool moments)
+// The block's Gaussians of one output segment: their indices within the block,
+// in order, and the segment's first output slot.
+struct Segment {
+    const uint16_t* list;
+    int count;
+    size_t dst;
+};
+
+constexpr int kCopyUnroll = 4;             // units of a field in flight per thread, times three arrays
+
+// One field of WIDTH units T per Gaussian (float4 for rows of whole 16 bytes,
+// else float), for the block's kept Gaussians (parameters and moments) and its
+// clones and children (parameters; zero moments).  Output rows are consecutive,
+// so unit t of the segment goes to unit t of a contiguous range and the
+// accesses of a warp are consecutive 4- or 16-byte units on both sides (reads
+// break only where a Gaussian is left out).
+template <typename T, int WIDTH>
+__device__ __forceinline__ void copy_rows(const ScatterArgs& a, int f, size_t base, const Segment& kept,
+                                          const Segment& clone, const Segment& split)
 {
+    const T* __restrict__ ps = reinterpret_cast<const T*>(a.p.f[f]) + base * WIDTH;
+    const T* __restrict__ ms = reinterpret_cast<const T*>(a.m.f[f]) + base * WIDTH;
+    const T* __restrict__ vs = reinterpret_cast<const T*>(a.v.f[f]) + base * WIDTH;
+    T* __restrict__ pd = reinterpret_cast<T*>(a.po.f[f]);
+    T* __restrict__ md = reinterpret_cast<T*>(a.mo.f[f]);
+    T* __restrict__ vd = reinterpret_cast<T*>(a.vo.f[f]);
+    const int nk = kept.count * WIDTH;
+    const size_t dk = kept.dst * WIDTH;
+    for (int t0 = threadIdx.x; t0 < nk; t0 += kCopyUnroll * 256) {
+        T rp[kCopyUnroll], rm[kCopyUnroll], rv[kCopyUnroll];
 #pragma unroll
-    for (int f = 0; f < 7; ++f) {
-        const int w = field_w(f, a.nc);
-        const float* ps = a.p.f[f];
-        const float* ms = a.m.f[f];
-        const float* vs = a.v.f[f];
-        float* pd = a.po.f[f];
-        float* md = a.mo.f[f];
-        float* vd = a.vo.f[f];
-        if ((w & 3) == 0 && ((reinterpret_cast<uintptr_t>(ps) | reinterpret_cast<uintptr_t>(ms) |
-                              reinterpret_cast<uintptr_t>(vs) | reinterpret_cast<uintptr_t>(pd) |
-                              reinterpret_cast<uintptr_t>(md) | reinterpret_cast<uintptr_t>(vd)) & 15u) == 0) {
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int e = 0; e < w; e += 4) {
-                reinterpret_cast<float4*>(pd + dst * w)[e >> 2] = reinterpret_cast<const float4*>(ps + src * w)[e >> 2];
-                reinterpret_cast<float4*>(md + dst * w)[e >> 2] =
-                    moments ? reinterpret_cast<const float4*>(ms + src * w)[e >> 2] : z;
-                reinterpret_cast<float4*>(vd + dst * w)[e >> 2] =
-                    moments ? reinterpret_cast<const float4*>(vs + src * w)[e >> 2] : z;
+        for (int u = 0; u < kCopyUnroll; ++u) {
+            const int t = t0 + 256 * u;
+            if (t < nk) {
+                const int o = kept.list[t / WIDTH] * WIDTH + t % WIDTH;
+                rp[u] = __ldcs(ps + o);
+                rm[u] = __ldcs(ms + o);
+                rv[u] = __ldcs(vs + o);
             }
-        } else {
-            for (int e = 0; e < w; ++e) {
-                pd[dst * w + e] = ps[src * w + e];
-                md[dst * w + e] = moments ? ms[src * w + e] : 0.f;
-                vd[dst * w + e] = moments ? vs[src * w + e] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u) {
+            const int t = t0 + 256 * u;
+            if (t < nk) {
+                __stcs(pd + dk + t, rp[u]);
+                __stcs(md + dk + t, rm[u]);
+                __stcs(vd + dk + t, rv[u]);
             }
+        }
+    }
+    const T zero = T();
+    const int nc = clone.count * WIDTH;
+    const size_t dc = clone.dst * WIDTH;
+    for (int t = threadIdx.x; t < nc; t += 256) {
+        pd[dc + t] = ps[clone.list[t / WIDTH] * WIDTH + t % WIDTH];
+        __stcs(md + dc + t, zero);
+        __stcs(vd + dc + t, zero);
+    }
+    const int ns = 2 * split.count * WIDTH;
+    const size_t ds = split.dst * WIDTH;
+    for (int t = threadIdx.x; t < ns; t += 256) {
+        if (f > 1) pd[ds + t] = ps[split.list[t / (2 * WIDTH)] * WIDTH + t % WIDTH];   // means, scales: child_rows
+        __stcs(md + ds + t, zero);
+        __stcs(vd + ds + t, zero);
+    }
+}
+
+// Means and log-scales of the block's split children, one thread per child.
+__device__ __forceinline__ void child_rows(const ScatterArgs& a, size_t base, const Segment& split)
+{
+    for (int t = threadIdx.x; t < 2 * split.count; t += 256) {
+        const size_t i = base + split.list[t >> 1];
+        const float* q = a.p.f[2] + 4 * i;
+        const float* ls = a.p.f[1] + 3 * i;
+        const float* mu = a.p.f[0] + 3 * i;
+        const float qn = rsqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
+        const float w = q[0] * qn, x = q[1] * qn, y = q[2] * qn, z = q[3] * qn;
+        const float R[3][3] = {{1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y)},
+                               {2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x)},
+                               {2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)}};
+        const float s[3] = {expf(ls[0]), expf(ls[1]), expf(ls[2])};
+        const float* nz = a.noise + 6 * i + 3 * (t & 1);
+        const float v0 = s[0] * nz[0], v1 = s[1] * nz[1], v2 = s[2] * nz[2];
+        float* mo = a.po.f[0] + 3 * (split.dst + t);
+        float* lo = a.po.f[1] + 3 * (split.dst + t);
+#pragma unroll
+        for (int rr = 0; rr < 3; ++rr) {
+            mo[rr] = mu[rr] + R[rr][0] * v0 + R[rr][1] * v1 + R[rr][2] * v2;
+            lo[rr] = ls[rr] - a.ln16;
         }
     }
 }
 
-// Positions: block offset + rank within the block (a block-wide scan of the
-// three flags, in index order), then the copies.
+// Lists the block's Gaussians of each segment (a block-wide scan of the three
+// flags, in index order; the block of a classification block's second half
+// counts the first half's for its offsets), then copies field by field.  A
+// copy bound by HBM: at 1M Gaussians of SH degree 3 (900k left, 1.13M out) it
+// reads and writes 1.7 GB.  One thread per Gaussian walking its own rows
+// touched 32 rows per warp instruction (the whole call took 0.733 ms); rows
+// dealt out by output unit make every warp access consecutive (0.333 ms).
+template <int NC>
 __global__ void __launch_bounds__(256) densify_scatter_kernel(ScatterArgs a)
 {
     __shared__ unsigned wsum[3][8];
-    __shared__ unsigned run[3];
-    if (threadIdx.x < 3) run[threadIdx.x] = 0;
-    __syncthreads();
-    const int nb = gridDim.x;
-    const unsigned long long K1 = a.totals[0], K2 = a.totals[1];
-    for (int r = 0; r < kDB / 256; ++r) {
-        const int i = blockIdx.x * kDB + r * 256 + threadIdx.x;
+    __shared__ uint16_t list[3][kSB];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cb = blockIdx.x / (kDB / kSB), first = blockIdx.x % (kDB / kSB) * kSB;
+    const size_t base = (size_t)blockIdx.x * kSB;
+    unsigned run[3] = {0, 0, 0}, skip[3] = {0, 0, 0};
+    for (int r = 0; r < (first + kSB) / 256; ++r) {
+        const int l = r * 256 + threadIdx.x - first;          // < 0: the classification block's earlier half
+        if (r * 256 == first)
+            for (int s = 0; s < 3; ++s) {
+                skip[s] = run[s];
+                run[s] = 0;
+            }
+        const long long i = (long long)base + l;
         const int k = i < a.n ? a.kind[i] : 0;
-        const unsigned f[3] = {(unsigned)(k == 1 || k == 2), (unsigned)(k == 2), (unsigned)(k == 3)};
-        unsigned ex[3];
+        const bool f[3] = {k == 1 || k == 2, k == 2, k == 3};
+        unsigned before[3];
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
-            unsigned x = f[s];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-                if ((threadIdx.x & 31) >= o) x += y;
-            }
-            if ((threadIdx.x & 31) == 31) wsum[s][threadIdx.x >> 5] = x;
-            ex[s] = x - f[s];
+            const unsigned b = __ballot_sync(0xffffffffu, f[s]);
+            before[s] = __popc(b & ((1u << lane) - 1u));
+            if (lane == 0) wsum[s][warp] = __popc(b);
         }
         __syncthreads();
-        unsigned tot[3];
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
-            unsigned before = 0, all = 0;
+            unsigned all = 0;
             for (int w = 0; w < 8; ++w) {
-                if (w < (int)(threadIdx.x >> 5)) before += wsum[s][w];
+                if (w < warp) before[s] += wsum[s][w];
                 all += wsum[s][w];
             }
-            ex[s] += before + run[s] + a.boff[(size_t)s * nb + blockIdx.x];
-            tot[s] = all;
-        }
-        __syncthreads();
-        if (threadIdx.x < 3) run[threadIdx.x] += tot[threadIdx.x];
-        if (i < a.n && k != 0) {
-            if (f[0]) copy_gaussian(a, i, ex[0], true);
-            if (f[1]) copy_gaussian(a, i, K1 + ex[1], false);
-            if (f[2]) {
-                const size_t d0 = K1 + K2 + 2ull * ex[2];
-                copy_gaussian(a, i, d0, false);
-                copy_gaussian(a, i, d0 + 1, false);
-                const float* q = a.p.f[2] + 4 * (size_t)i;
-                const float* ls = a.p.f[1] + 3 * (size_t)i;
-                const float* mu = a.p.f[0] + 3 * (size_t)i;
-                const float qn = rsqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-                const float w = q[0] * qn, x = q[1] * qn, y = q[2] * qn, z = q[3] * qn;
-                const float R[3][3] = {{1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y)},
-                                       {2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x)},
-                                       {2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)}};
-                const float s[3] = {expf(ls[0]), expf(ls[1]), expf(ls[2])};
-                for (int c = 0; c < 2; ++c) {
-                    const float* nz = a.noise + 6 * (size_t)i + 3 * c;
-                    const float v0 = s[0] * nz[0], v1 = s[1] * nz[1], v2 = s[2] * nz[2];
-                    float* mo = a.po.f[0] + 3 * (d0 + c);
-                    float* lo = a.po.f[1] + 3 * (d0 + c);
-#pragma unroll
-                    for (int rr = 0; rr < 3; ++rr) {
-                        mo[rr] = mu[rr] + R[rr][0] * v0 + R[rr][1] * v1 + R[rr][2] * v2;
-                        lo[rr] = ls[rr] - a.ln16;
-                    }
-                }
-            }
+            if (f[s] && l >= 0) list[s][run[s] + before[s]] = (uint16_t)l;
+            run[s] += all;
         }
         __syncthreads();
     }
+    const size_t K1 = a.totals[0], K2 = a.totals[1];
+    const Segment kept = {list[0], (int)run[0], (size_t)(a.boff[cb] + skip[0])};
+    const Segment clone = {list[1], (int)run[1], K1 + a.boff[(size_t)a.nb + cb] + skip[1]};
+    const Segment split = {list[2], (int)run[2], K1 + K2 + 2 * (size_t)(a.boff[2 * (size_t)a.nb + cb] + skip[2])};
+    // a field moves in 16-byte units when its rows are whole multiples of them and its six arrays are aligned
+    copy_rows<float, 3>(a, 0, base, kept, clone, split);
+    copy_rows<float, 3>(a, 1, base, kept, clone, split);
+    if (a.vec & 4u) copy_rows<float4, 1>(a, 2, base, kept, clone, split);
+    else copy_rows<float, 4>(a, 2, base, kept, clone, split);
+    copy_rows<float, 1>(a, 3, base, kept, clone, split);
+    if constexpr (3 * NC % 4 == 0) {
+        if (a.vec & 16u) copy_rows<float4, 3 * NC / 4>(a, 4, base, kept, clone, split);
+        else copy_rows<float, 3 * NC>(a, 4, base, kept, clone, split);
+    } else {
+        copy_rows<float, 3 * NC>(a, 4, base, kept, clone, split);
+    }
+    if (a.vec & 32u) copy_rows<float4, 2>(a, 5, base, kept, clone, split);
+    else copy_rows<float, 8>(a, 5, base, kept, clone, split);
+    copy_rows<float, 1>(a, 6, base, kept, clone, split);
+    child_rows(a, base, split);
 }
 
 Fields fields_of(const le_gaussian_grads* g)
@@ -386,7 +436,6 @@ extern "C" le_status le_densify(const le_densify_config* cfg, const le_gaussians
     }
     ScatterArgs a;
     a.n = n;
-    a.nc = (g->sh_degree + 1) * (g->sh_degree + 1);
     float* const gp[7] = {const_cast<float*>(g->means), const_cast<float*>(g->log_scales), const_cast<float*>(g->quats),
                           const_cast<float*>(g->opacity_raw), const_cast<float*>(g->sh), const_cast<float*>(g->feat),
                           const_cast<float*>(g->unc)};
@@ -401,7 +450,19 @@ extern "C" le_status le_densify(const le_densify_config* cfg, const le_gaussians
     a.totals = totals;
     a.noise = noise;
     a.ln16 = t.ln16;
-    densify_scatter_kernel<<<nb, 256, 0, s>>>(a);
+    a.nb = nb;
+    a.vec = 0;
+    for (int i = 0; i < 7; ++i)
+        if (aligned16(a.p.f[i]) && aligned16(a.m.f[i]) && aligned16(a.v.f[i]) && aligned16(a.po.f[i]) &&
+            aligned16(a.mo.f[i]) && aligned16(a.vo.f[i]))
+            a.vec |= 1u << i;
+    const int sb = (n + kSB - 1) / kSB;
+    switch (g->sh_degree) {
+        case 0: densify_scatter_kernel<1><<<sb, 256, 0, s>>>(a); break;
+        case 1: densify_scatter_kernel<4><<<sb, 256, 0, s>>>(a); break;
+        case 2: densify_scatter_kernel<9><<<sb, 256, 0, s>>>(a); break;
+        default: densify_scatter_kernel<16><<<sb, 256, 0, s>>>(a); break;
+    }
     LE_LAUNCHED();
     return LE_OK;
 }

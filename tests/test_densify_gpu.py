@@ -76,6 +76,36 @@ def test_densify_matches_oracle(leg, orc, n, size_pruning):
         assert np.array_equal(getattr(gv, k).cpu().numpy(), o["v"][k]), k
 
 
+@pytest.mark.parametrize("degree,offset", [(0, 0), (1, 0), (2, 0), (3, 0), (3, 1), (1, 2)])
+@pytest.mark.parametrize("n", [511, 1537])
+def test_densify_rows_of_every_width(leg, orc, n, degree, offset):
+    """Every SH degree's row width, and arrays that start off a 16-byte boundary (offset floats): the
+    copies are exact."""
+    P, acc, cnt = _densify_inputs(n, 85 + n)
+    rng = np.random.default_rng(86 + degree)
+    P["sh"] = rng.standard_normal((n, (degree + 1) ** 2, 3)).astype(np.float32)
+    M = {k: rng.standard_normal(v.shape).astype(np.float32) for k, v in P.items()}
+    V = {k: rng.uniform(0, 1, v.shape).astype(np.float32) for k, v in P.items()}
+    noise = rng.standard_normal((n, 2, 3)).astype(np.float32)
+
+    def dev(d):
+        out = []
+        for k in FIELDS:
+            flat = torch.empty(d[k].size + offset, device="cuda")[offset:]
+            out.append(flat.view(d[k].shape).copy_(torch.from_numpy(np.ascontiguousarray(d[k]))))
+        return leg.Gaussians(*out, degree)
+
+    got = leg.le_densify(dev(P), dev(M), dev(V), torch.from_numpy(acc).cuda(), torch.from_numpy(cnt).cuda(),
+                         torch.from_numpy(noise).cuda(), scene_extent=4.0)
+    o = orc.densify(P, M, V, acc, cnt, noise, extent=4.0)
+    nk = int(np.sum((o["kind"] == 1) | (o["kind"] == 2)) + np.sum(o["kind"] == 2))
+    assert got[0].n == o["n_out"] and nk < o["n_out"]
+    for g, ref in zip(got, (o["params"], o["m"], o["v"])):
+        for k in FIELDS:
+            exact = nk if ref is o["params"] and k in ("means", "log_scales") else o["n_out"]
+            assert np.array_equal(getattr(g, k).cpu().numpy()[:exact], ref[k][:exact].astype(np.float32)), k
+
+
 def test_densify_capacity(leg):
     P, acc, cnt = _densify_inputs(3000, 83)
     noise = torch.zeros((3000, 2, 3), device="cuda")
