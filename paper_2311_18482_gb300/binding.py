@@ -195,14 +195,9 @@ def reset_launch_count():
 
 # ---------------------------------------------------------------------------
 def camera_struct(cam) -> LeCamera:
-    c = LeCamera()
-    c.view[:] = [float(v) for v in cam.view]
-    c.campos[:] = [float(v) for v in cam.campos]
-    c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
-    c.width, c.height = int(cam.W), int(cam.H)
-    c.near_z = float(cam.near)
-    c.bg[:] = [float(v) for v in cam.bg]
-    return c
+    floats = lambda a: (C.c_float * len(a))(*(a.tolist() if hasattr(a, "tolist") else map(float, a)))
+    return LeCamera(floats(cam.view), floats(cam.campos), float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy),
+                    int(cam.W), int(cam.H), float(cam.near), floats(cam.bg))
 
 
 @dataclass
@@ -228,11 +223,15 @@ class Gaussians:
                          f(scene.feat), f(scene.unc), scene.sh_degree)
 
     def struct(self) -> LeGaussians:
-        s = LeGaussians()
-        s.n, s.sh_degree = self.n, self.sh_degree
-        for k in ("means", "log_scales", "quats", "opacity_raw", "sh", "feat", "unc"):
-            setattr(s, k, getattr(self, k).data_ptr())
-        return s
+        return LeGaussians(self.n, self.sh_degree, *self._ptrs())
+
+    def _ptrs(self):
+        return (self.means.data_ptr(), self.log_scales.data_ptr(), self.quats.data_ptr(),
+                self.opacity_raw.data_ptr(), self.sh.data_ptr(), self.feat.data_ptr(), self.unc.data_ptr())
+
+    def empty_like(self) -> "Gaussians":
+        return Gaussians(*(torch.empty_like(getattr(self, k)) for k in
+                           ("means", "log_scales", "quats", "opacity_raw", "sh", "feat", "unc")), self.sh_degree)
 
     def zeros_like(self) -> "Gaussians":
         return Gaussians(*(torch.zeros_like(getattr(self, k)) for k in
@@ -240,10 +239,7 @@ class Gaussians:
 
 
 def grads_struct(g: Gaussians) -> LeGaussianGrads:
-    s = LeGaussianGrads()
-    for k in ("means", "log_scales", "quats", "opacity_raw", "sh", "feat", "unc"):
-        setattr(s, k, getattr(g, k).data_ptr())
-    return s
+    return LeGaussianGrads(*g._ptrs())
 
 
 @dataclass
@@ -267,10 +263,7 @@ class Projected:
                          torch.empty((n, 8), dtype=torch.float32, device=device))
 
     def struct(self) -> LeProjected:
-        s = LeProjected()
-        for k in _PROJ_FIELDS:
-            setattr(s, k, getattr(self, k).data_ptr())
-        return s
+        return LeProjected(*(getattr(self, k).data_ptr() for k in _PROJ_FIELDS))
 
 
 # ---------------------------------------------------------------------------
@@ -407,7 +400,7 @@ def le_bin_render_fwd(cam, proj: Projected, buffers: BinSortBuffers | None = Non
 
 def le_render_bwd(cam, g: Gaussians, proj: Projected, ids, ranges, img: Image, dL_drgb, dL_dfeat, dL_dunc,
                   grads: Gaussians | None = None, grad2d=None):
-    grads = grads or g.zeros_like()
+    grads = grads or g.empty_like()          # every element is written
     grad2d = grad2d if grad2d is not None else torch.empty((g.n, SPLAT_STRIDE), dtype=torch.float32,
                                                            device=g.means.device)
     cs, gs, ps, os_ = camera_struct(cam), g.struct(), proj.struct(), grads_struct(grads)
@@ -447,7 +440,7 @@ def le_render_bwd_screen(cam, g: Gaussians, proj: Projected, ids, ranges, img: I
 
 def le_project_bwd(cam, g: Gaussians, proj: Projected, grad2d, grads: Gaussians | None = None) -> Gaussians:
     """Projection half of le_render_bwd: parameter gradients from grad2d."""
-    grads = grads or g.zeros_like()
+    grads = grads or g.empty_like()          # every element is written
     cs, gs, ps, os_ = camera_struct(cam), g.struct(), proj.struct(), grads_struct(grads)
     _check(load().le_project_bwd(C.byref(cs), C.byref(gs), C.byref(ps), _ptr(grad2d), C.byref(os_), _stream()))
     return grads
@@ -749,10 +742,15 @@ class _Rasterize(torch.autograd.Function):
         k_cap = max(16 * g.n, int(1.25 * hint) + 1024) if own and hint is not None else None
         ids, ranges, K, img = le_bin_render_fwd(cam, proj, BinSortBuffers() if own else buffers, k_cap=k_cap)
         _K_HINT[means.device] = K
+        ctx.cam, ctx.g, ctx.proj = cam, g, proj
+        # Of the outputs only T (not differentiable) is kept: a differentiable output held here would tie
+        # itself, through its grad_fn, to this node -- a cycle the collector cannot see, which kept every
+        # view's images, lists and projection (0.4 GB at 1M Gaussians) alive for good.
+        ctx.T, ctx.n_contrib = img.T, img.n_contrib
         # buffers the caller reuses may be overwritten by a later forward before this backward
-        ctx.cam, ctx.g, ctx.proj, ctx.img = cam, g, proj, img
         ctx.ids, ctx.ranges = (ids, ranges) if own else (ids.clone(), ranges.clone())
         ctx.mark_non_differentiable(img.T)
+        ctx.set_materialize_grads(False)     # no zero image for T or for an output the loss does not use
         return img.rgb, img.feat, img.unc, img.T
 
     @staticmethod
@@ -763,7 +761,8 @@ class _Rasterize(torch.autograd.Function):
         d_rgb = d_rgb if d_rgb is not None else z(3, H, W)
         d_feat = d_feat if d_feat is not None else z(8, H, W)
         d_unc = d_unc if d_unc is not None else z(H, W)
-        grads, _ = le_render_bwd(ctx.cam, ctx.g, ctx.proj, ctx.ids, ctx.ranges, ctx.img, d_rgb, d_feat, d_unc)
+        img = Image(None, None, None, ctx.T, ctx.n_contrib)
+        grads, _ = le_render_bwd(ctx.cam, ctx.g, ctx.proj, ctx.ids, ctx.ranges, img, d_rgb, d_feat, d_unc)
         return (grads.means, grads.log_scales, grads.quats, grads.opacity_raw, grads.sh, grads.feat, grads.unc,
                 None, None, None)
 

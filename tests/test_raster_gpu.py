@@ -122,6 +122,28 @@ def test_autograd_function(leg, orc):
     assert rel_err(to_np(params[6].grad), g2["unc"]) < 1e-4
 
 
+def test_autograd_memory_is_given_back(leg):
+    """A view's buffers go once its outputs and graph are dropped, without a garbage collection; an
+    output the loss leaves out gets a zero gradient."""
+    c = synth.config("c1", n=800, W=64, H=64)
+    params = [torch.from_numpy(getattr(c["scene"], k)).cuda().requires_grad_(True)
+              for k in ("means", "log_scales", "quats", "opacity_raw", "sh", "feat", "unc")]
+
+    def view():
+        rgb = leg.rasterize(*params, c["camera"], c["scene"].sh_degree)[0]
+        return torch.autograd.grad(rgb.sum(), params)
+
+    grads = view()
+    assert not grads[5].any() and not grads[6].any() and grads[4].any()
+    del grads
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    for _ in range(3):
+        view()
+    torch.cuda.synchronize()
+    assert torch.cuda.memory_allocated() == before
+
+
 def test_degenerate_scenes(leg, orc):
     # all Gaussians behind the camera: K = 0, background everywhere, zero gradients
     c = synth.config("c1", n=50, W=40, H=24)
