@@ -11,8 +11,9 @@
 // ordered by depth, ties by Gaussian index.  It is computed without sorting the
 // K copies at all:
 //   1. e[i] = bits(depth_i) << 32 | i          (culled: 0xFFFFFFFF, sorted last)
-//   2. stable LSD radix sort of e on bits 32..63 (4 passes over the N Gaussians,
-//      each count / scan / scatter, see depth_sort)
+//   2. stable order of e by bits 32..63: up to kRankMax Gaussians by counting
+//      (depth_rank_kernel), else an LSD radix sort (4 passes over the N
+//      Gaussians, each count / scan / scatter, see depth_sort)
 //   3. split the depth-sorted Gaussians into chunks; per chunk, the number of
 //      copies in every tile from per-row difference arrays of the row spans
 //   4. one exclusive scan of those counts in tile-major order: entry (t, c) is
@@ -111,7 +112,6 @@ __global__ void __launch_bounds__(kThreads) scan_apply_kernel(In in, int n, uint
             uint32_t t = 0;
             for (int w = 0; w < kWarps; ++w) t += ws[w];
             s_off = t;
-            if (blockIdx.x == gridDim.x - 1) *total = t + partials[blockIdx.x];
         }
         __syncthreads();
     }
@@ -129,7 +129,9 @@ __global__ void __launch_bounds__(kThreads) scan_apply_kernel(In in, int n, uint
         v[k] = sm[j + (j >> 5)];
         s += v[k];
     }
-    uint32_t run = block_exclusive_scan(s, ws, nullptr) + s_off;
+    uint32_t own = 0;
+    uint32_t run = block_exclusive_scan(s, ws, &own) + s_off;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = s_off + own;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
         const int j = threadIdx.x * kItems + k;
@@ -152,8 +154,10 @@ le_status exclusive_scan(In in, int n, uint32_t* out, uint32_t* partials, uint32
         set_error("scan of %d elements exceeds the supported size", n);
         return LE_ERR_CAPACITY;
     }
-    scan_reduce_kernel<In><<<nb, kThreads, 0, s>>>(in, n, partials);
-    LE_LAUNCHED();
+    if (nb > 1) {               // one block has no blocks before it
+        scan_reduce_kernel<In><<<nb, kThreads, 0, s>>>(in, n, partials);
+        LE_LAUNCHED();
+    }
     scan_apply_kernel<In><<<nb, kThreads, 0, s>>>(in, n, out, partials, total);
     LE_LAUNCHED();
     return LE_OK;
@@ -374,6 +378,66 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64
             gather.dell[2 * (size_t)p + 1] = e1;
         }
     }
+}
+
+// The whole depth order of at most kRankMax Gaussians in one launch: an
+// element's position is the number of elements that sort before it, counted
+// directly.  Eight threads per element, each over every eighth group of four
+// keys of a shared-memory tile that all of the block's elements read together.
+// n^2 compares (0.27 G at 16,384) replace a memset and twelve dependent
+// launches that leave most of the chip idle at this size: le_bin_sort on 2,000 /
+// 8,192 / 16,384 Gaussians takes 69 / 97 / 121 us against 145 / 170 / 170 us,
+// and the compares, growing with n^2, would meet the radix passes near 25,000.
+constexpr int kRankMax = 16384, kRankThreads = 256, kRankKeys = 2048;
+
+__global__ void __launch_bounds__(kRankThreads) depth_rank_kernel(int n, const float* __restrict__ depth,
+                                                                  uint64_t* __restrict__ out, SortGather gather)
+{
+    __shared__ __align__(16) uint32_t keys[kRankKeys];
+    constexpr int kElems = kRankThreads / 8;
+    const int part = threadIdx.x & 7, i0 = blockIdx.x * kElems, i = i0 + (threadIdx.x >> 3);
+    const auto key = [&](int j) { return gather.tiles[j] > 0 ? __float_as_uint(depth[j]) : 0xFFFFFFFFu; };
+    const uint32_t mine = i < n ? key(i) : 0u;
+    uint32_t rank = 0;
+    for (int t0 = 0; t0 < n; t0 += kRankKeys) {
+        __syncthreads();
+        // past the end: a key that is below none, at an index above all
+        for (int j = threadIdx.x; j < kRankKeys; j += kRankThreads) keys[j] = t0 + j < n ? key(t0 + j) : 0xFFFFFFFFu;
+        __syncthreads();
+        const int groups = min(kRankKeys, (n - t0 + 31) / 32 * 32) / 4;
+        const uint4* k4 = reinterpret_cast<const uint4*>(keys);
+        // equal keys keep index order: they count when the tile lies before the
+        // block's elements, not when it lies behind, by index in between
+        if (t0 + kRankKeys <= i0) {
+            for (int q = part; q < groups; q += 8) {
+                const uint4 k = k4[q];
+                rank += (k.x <= mine) + (k.y <= mine) + (k.z <= mine) + (k.w <= mine);
+            }
+        } else if (t0 >= i0 + kElems) {
+            for (int q = part; q < groups; q += 8) {
+                const uint4 k = k4[q];
+                rank += (k.x < mine) + (k.y < mine) + (k.z < mine) + (k.w < mine);
+            }
+        } else {
+            for (int q = part; q < groups; q += 8) {
+                const uint4 k = k4[q];
+                const int j = t0 + 4 * q;
+                rank += (k.x < mine || (k.x == mine && j < i)) + (k.y < mine || (k.y == mine && j + 1 < i)) +
+                        (k.z < mine || (k.z == mine && j + 2 < i)) + (k.w < mine || (k.w == mine && j + 3 < i));
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (i >= n) return;
+    const bool seen = gather.tiles[i] > 0;
+    if (part == 0) out[rank] = ((uint64_t)mine << 32) | (uint32_t)i;
+    if (part == 1)
+        reinterpret_cast<uint2*>(gather.drect)[rank] =
+            seen ? reinterpret_cast<const uint2*>(gather.rect)[i] : make_uint2(0u, 0u);
+    if (part == 2 || part == 3)
+        gather.dell[2 * (size_t)rank + part - 2] =
+            seen ? gather.ell[2 * (size_t)i + part - 2] : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // Tiles [xl, xr) of rectangle row ty that the tile ellipse {e0, e1} reaches.
@@ -697,8 +761,7 @@ SortWs sort_ws_layout(char* base, int32_t n)
 // The four passes (pass 0's counts are in w.counts and w.sort_state, counted
 // by depth_elems_kernel).  Result in *cur; the rectangles and tile ellipses in
 // depth order in w.drect and w.dell.
-le_status depth_sort(uint64_t*& cur, uint64_t*& alt, int n, const SortWs& w, const int* tiles, const ushort4* rect,
-                     const float4* ell, cudaStream_t s)
+le_status depth_sort(uint64_t*& cur, uint64_t*& alt, int n, const SortWs& w, const SortGather& gather, cudaStream_t s)
 {
     const int nt = sort_tiles(n), row = sort_row(n);
     for (int q = 0; q < kSortPasses; ++q) {
@@ -710,9 +773,8 @@ le_status depth_sort(uint64_t*& cur, uint64_t*& alt, int n, const SortWs& w, con
         }
         sort_rowscan_kernel<<<256 / 8, 256, 0, s>>>(w.counts, nt, row, totals);
         LE_LAUNCHED();
-        SortGather g{};
-        if (q == kSortPasses - 1) g = SortGather{tiles, rect, ell, w.drect, w.dell};
-        sort_scatter_kernel<<<nt, kSortThreads, 0, s>>>(cur, alt, n, shift, w.counts, row, g);
+        sort_scatter_kernel<<<nt, kSortThreads, 0, s>>>(cur, alt, n, shift, w.counts, row,
+                                                        q == kSortPasses - 1 ? gather : SortGather{});
         LE_LAUNCHED();
         uint64_t* t = cur;
         cur = alt;
@@ -773,16 +835,22 @@ le_status bin_prepare(const le_camera* cam, int32_t n, const float* depth, const
     }
 
     // 1-2: sort the Gaussians by depth (stable: equal depths keep index order; culled last)
-    LE_CUDA(cudaMemsetAsync(w.sort_state, 0, 4 * sort_state_words(n), s));
-    depth_elems_kernel<<<sort_tiles(n), kSortThreads, 0, s>>>(n, depth, tiles_touched, w.eA, w.counts, sort_row(n),
-                                                              w.sort_state);
-    LE_LAUNCHED();
-    cur = w.eA;
-    uint64_t* alt = w.eB;
     // 3: (with the last pass) rectangles and ellipses in depth order
-    if ((st = depth_sort(cur, alt, n, w, tiles_touched, reinterpret_cast<const ushort4*>(rect),
-                         reinterpret_cast<const float4*>(tile_ellipse), s)) != LE_OK)
-        return st;
+    const SortGather gather{tiles_touched, reinterpret_cast<const ushort4*>(rect),
+                            reinterpret_cast<const float4*>(tile_ellipse), w.drect, w.dell};
+    cur = w.eA;
+    if (n <= kRankMax) {
+        constexpr int kElems = kRankThreads / 8;
+        depth_rank_kernel<<<(n + kElems - 1) / kElems, kRankThreads, 0, s>>>(n, depth, cur, gather);
+        LE_LAUNCHED();
+    } else {
+        LE_CUDA(cudaMemsetAsync(w.sort_state, 0, 4 * sort_state_words(n), s));
+        depth_elems_kernel<<<sort_tiles(n), kSortThreads, 0, s>>>(n, depth, tiles_touched, w.eA, w.counts, sort_row(n),
+                                                                  w.sort_state);
+        LE_LAUNCHED();
+        uint64_t* alt = w.eB;
+        if ((st = depth_sort(cur, alt, n, w, gather, s)) != LE_OK) return st;
+    }
     // copies per (tile, chunk of depth-sorted Gaussians)
     const size_t diff_smem = sizeof(int4) * (((size_t)(TX + 1) * TY + 3) / 4);
     if (diff_smem > 48 * 1024)

@@ -169,6 +169,22 @@ def test_degenerate_scenes(leg, orc):
     assert K == 0 and np.all(to_np(img.T) == 1)
 
 
+@pytest.mark.parametrize("n", [1, 31, 33, 2047, 2049, 16384, 16385])
+def test_binning_order_on_both_sorts(leg, orc, n):
+    """Few Gaussians are ordered by counting, more by radix passes: with every depth shared by two or
+    more Gaussians, the lists and ranges equal the oracle's stable sort."""
+    c = synth.config("c1", n=n, W=64, H=48)
+    sc, cam = c["scene"], c["camera"]
+    sc.means[:] = sc.means[np.arange(n) // 2 % 700]
+    sc.log_scales -= 1.0
+    g = leg.Gaussians.from_scene(sc)
+    ids, ranges, K, _ = leg.le_bin_sort(cam, leg.le_preprocess(g, cam))
+    ref = orc.forward(sc, cam)
+    assert K == len(ref["vals"])
+    assert np.array_equal(ids.cpu().numpy().view(np.uint32), ref["vals"])
+    assert np.array_equal(ranges.cpu().numpy().view(np.uint32).reshape(-1), np.asarray(ref["ranges"]).reshape(-1))
+
+
 def test_deterministic_binning(leg):
     c = synth.config("c2", n=50000, W=320, H=240)
     sc, cam = c["scene"], c["camera"]
