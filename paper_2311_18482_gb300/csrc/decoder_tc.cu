@@ -84,9 +84,10 @@ struct Front {
     uint32_t lane;     // this warp's TMEM lane field
     int tid;           // row of the tile (TMEM lane) this thread serves
     int bar_id, nthreads;
+    bool issuer;       // the warp that issues this group's MMAs (warp-uniform)
     int half, nhalf;
     float4* xch;       // [nhalf][128] (nhalf > 1 only)
-    // W3s reloaded by a bulk copy (thread 0 only): the third layer's MMAs wait
+    // W3s reloaded by a bulk copy (the issuing warp): the third layer's MMAs wait
     // for it first
     uint64_t* w3bar = nullptr;
     uint32_t w3phase = 0;
@@ -150,7 +151,7 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
         sbuf_store8(f.X1, f.tid, 8, v);
     }
     wg_publish(f);
-    if (f.tid == 0 && f.half == 0) {
+    if (f.issuer && elect_one()) {
         mma(f.tw, kdesc(f.X1, 0, 0), kdesc(f.W1s, 0, 0), idesc_bf16(kH1, false, false), 0);
         commit(f.mbar);
     }
@@ -165,7 +166,7 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
         sbuf_store8(f.H1, f.tid, c + 8, v + 8);
     }
     wg_publish(f);
-    if (f.tid == 0 && f.half == 0) {
+    if (f.issuer && elect_one()) {
 #pragma unroll
         for (int s = 0; s < kH1 / 16; ++s)
             mma(f.tw, kdesc(f.H1, 0, 16 * s), kdesc(f.W2s, 0, 16 * s), idesc_bf16(kH2, false, false), s > 0);
@@ -181,16 +182,19 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
         sbuf_store8(f.H2, f.tid, c + 8, v + 8);
     }
     wg_publish(f);
-    if (f.tid == 0 && f.half == 0) {
+    if (f.issuer) {
         if (f.w3pending) {
             if (!mbar_wait(f.w3bar, f.w3phase)) atomicExch(&g_tc_error, 1);
             f.w3phase ^= 1u;
             f.w3pending = false;
         }
+        if (elect_one()) {
+            const uint32_t id = idesc_bf16(a.ncb, false, false);
 #pragma unroll
-        for (int s = 0; s < kH2 / 16; ++s)
-            mma(f.tw, kdesc(f.H2, 0, 16 * s), kdesc(f.W3s, 0, 16 * s), idesc_bf16(a.ncb, false, false), s > 0);
-        commit(f.mbar);
+            for (int s = 0; s < kH2 / 16; ++s)
+                mma(f.tw, kdesc(f.H2, 0, 16 * s), kdesc(f.W3s, 0, 16 * s), id, s > 0);
+            commit(f.mbar);
+        }
     }
     return wg_wait(f);
 }
@@ -292,7 +296,7 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
     extern __shared__ __align__(1024) unsigned char sm[];
     Front f;
     unsigned char* p = load_weights(sm, a, f);
-    const int wg = threadIdx.x >> 7;
+    const int warp = (int)warp_uniform(threadIdx.x >> 5), wg = warp >> 2;
     unsigned char* q = p + wg * kFwdWgBytes;
     f.X1 = SBuf{q, 16};
     f.H1 = SBuf{q + sbuf_bytes(128, 16), 64};
@@ -303,6 +307,7 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
     f.phase = 0;
     f.tid = threadIdx.x & 127;
     f.bar_id = 1 + wg;
+    f.issuer = (warp & 3) == 0;
     f.nthreads = NWG == 1 ? (int)blockDim.x : 128;
     f.half = 0;
     f.nhalf = 1;
@@ -314,7 +319,7 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t*>(slot);
+    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
     f.tw = tbase + 256 * wg;
     f.lane = (uint32_t)(32 * (f.tid >> 5)) << 16;
 
@@ -454,7 +459,7 @@ __device__ __forceinline__ void train_stage(int st, int ncb, uint32_t w1, uint32
     }
 }
 
-// The MMA thread: tile pairs in order, stage by stage, slot 0 then slot 1.
+// The MMA warp: tile pairs in order, stage by stage, slot 0 then slot 1.
 __device__ __forceinline__ bool train_mma_loop(int ncb, const Front& f, uint32_t e, uint32_t slots,
                                                uint64_t* ready, uint64_t* done, uint32_t tb, int ntiles)
 {
@@ -466,12 +471,14 @@ __device__ __forceinline__ bool train_mma_loop(int ncb, const Front& f, uint32_t
         const int nsl = t0 + (int)gridDim.x < ntiles ? 2 : 1;
         for (int st = 0; st < 6; ++st)
             for (int s = 0; s < nsl; ++s) {
-                if (!mbar_wait(ready + s, ph[s])) return false;
+                if (!warp_agree(mbar_wait(ready + s, ph[s]))) return false;
                 ph[s] ^= 1u;
                 fence_after();
-                train_stage(st, ncb, opaque(w1), opaque(w2), opaque(w3), opaque(e), opaque(slots + kSlotBytes * s),
-                            tb + 128u * s, tb, it == 0 && s == 0);
-                commit(done + s);
+                if (elect_one()) {
+                    train_stage(st, ncb, w1, w2, w3, e, slots + kSlotBytes * s, tb + 128u * s, tb, it == 0 && s == 0);
+                    commit(done + s);
+                }
+                __syncwarp();
             }
     }
     return true;
@@ -774,7 +781,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) dec_train_kernel(DecArgs a)
     uint64_t* done = ready + 2;
     uint64_t* fin = ready + 4;
     uint32_t* slot_addr = reinterpret_cast<uint32_t*>(ready + 5);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     // the slots start zeroed (padding columns feed MMA rows that are never read,
     // and must hold finite values); E has ones in columns 8 and 17
     for (size_t i = threadIdx.x; i < 2 * train_slot_bytes() / 16; i += blockDim.x)
@@ -798,17 +805,15 @@ __global__ void __launch_bounds__(kTrainThreads, 1) dec_train_kernel(DecArgs a)
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tb = *reinterpret_cast<volatile uint32_t*>(slot_addr);
+    const uint32_t tb = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot_addr));
     const int ntiles = (a.P + 127) / 128;
     bool ok = true;
     float acc_ce = 0.f, acc_u = 0.f, acc_l1 = 0.f;
     if (warp == 16) {
-        if (lane == 0) {
-            ok = train_mma_loop(a.ncb, f, smem_u32(E.p), slots_a, ready, done, tb, ntiles);
-            if (ok) {
-                commit(fin);
-                ok = mbar_wait(fin, 0);
-            }
+        ok = train_mma_loop(a.ncb, f, smem_u32(E.p), slots_a, ready, done, tb, ntiles);
+        if (ok) {
+            if (elect_one()) commit(fin);
+            ok = mbar_wait(fin, 0);
         }
     } else {
         EpiCtx e;
@@ -928,7 +933,9 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
     f.tid = tid & 127;
     f.bar_id = 0;
     f.nthreads = blockDim.x;
-    f.half = tid >> 7;
+    const int warp = (int)warp_uniform(threadIdx.x >> 5);
+    f.half = warp >> 2;
+    f.issuer = warp == 0;
     f.nhalf = kQueryParts;
     f.w3bar = mbar + 4;
     if (tid == 0) {
@@ -940,7 +947,7 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t*>(slot);
+    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
     f.tw = tbase;
     f.lane = (uint32_t)(32 * ((tid >> 5) & 3)) << 16;
     const int row = f.tid;
@@ -948,14 +955,16 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
     my_cols(f, a.ncb, c0, c1);                  // this part's class columns
     const int nch = a.ncb / 64;                 // G chunks (64 K-columns each)
     const int nlow = nch < 2 ? nch : 2, nup = nch - nlow;
-    // loads in flight (thread 0 only): chunks 0-1 (once), chunks 2-3 (per tile)
+    // loads in flight (the issuing warp): chunks 0-1 (once), chunks 2-3 (per tile)
     bool low_pending = false, up_pending = false;
     uint32_t up_phase = 0u;
     const int ntiles = (a.P + 127) / 128;
     bool ok = true;
-    if (tid == 0 && blockIdx.x < ntiles) {
-        mbar_expect_tx(mbar + 1, nlow * chunk_bytes);
-        bulk_g2s(g_own, a.G_img, nlow * chunk_bytes, mbar + 1);
+    if (f.issuer && (int)blockIdx.x < ntiles) {
+        if (elect_one()) {
+            mbar_expect_tx(mbar + 1, nlow * chunk_bytes);
+            bulk_g2s(g_own, a.G_img, nlow * chunk_bytes, mbar + 1);
+        }
         low_pending = true;
     }
     float xf[8];                                // this tile's R_s, loaded a tile ahead (part 0)
@@ -965,9 +974,11 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
         const bool valid = px < a.P;
         if (!mlp_forward_x(f, a, xf)) break;
         // the third layer's MMAs have read W3: chunks 2-3 of G take its place
-        if (tid == 0 && nup > 0) {
-            mbar_expect_tx(mbar + 2, nup * chunk_bytes);
-            bulk_g2s(f.W3s.p, a.G_img + 2 * (size_t)chunk_bytes, nup * chunk_bytes, mbar + 2);
+        if (f.issuer && nup > 0) {
+            if (elect_one()) {
+                mbar_expect_tx(mbar + 2, nup * chunk_bytes);
+                bulk_g2s(f.W3s.p, a.G_img + 2 * (size_t)chunk_bytes, nup * chunk_bytes, mbar + 2);
+            }
             up_pending = true;
         }
         if (f.half == 0) {
@@ -1000,9 +1011,15 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
         wg_publish(f);
         // p . (S_c [q; n]) into [0, 16), p^T G into [256, 256 + ncb), all chunks in one round
         bool tmo = false;
-        if (tid == 0) {
-            for (int s = 0; s < a.ncb / 16; ++s)
-                mma(tbase, kdesc(Ps, 0, 16 * s), kdesc(Aqs, 0, 16 * s), idesc_bf16(16, false, false), s > 0);
+        if (f.issuer) {
+            const uint64_t pd = kdesc(Ps, 0, 0), qd = kdesc(Aqs, 0, 0);
+            const uint32_t id = idesc_bf16(a.ncb, false, false);
+            for (int kc = 0; kc < nch; ++kc)
+                if (elect_one())
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        mma(tbase, pd + 64 * kc + 16 * k, qd + 64 * kc + 16 * k, idesc_bf16(16, false, false),
+                            kc > 0 || k > 0);
             if (low_pending) {
                 if (!mbar_wait(mbar + 1, 0u)) tmo = true;
                 low_pending = false;
@@ -1013,20 +1030,24 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
                     up_phase ^= 1u;
                     up_pending = false;
                 }
-                for (int k = 0; k < 4; ++k)
-                    mma(tbase + kTG, kdesc(Ps, 0, 64 * kc + 16 * k), kdesc(g_chunk(kc), 0, 16 * k),
-                        idesc_bf16(a.ncb, false, false), kc > 0 || k > 0);
+                const uint64_t gd = kdesc(g_chunk(kc), 0, 0);
+                if (elect_one())
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        mma(tbase + kTG, pd + 64 * kc + 16 * k, gd + 16 * k, id, kc > 0 || k > 0);
             }
-            commit(f.mbar);
+            if (elect_one()) commit(f.mbar);
         }
         if (!wg_wait(f) || bar_any(0, blockDim.x, tmo)) {
             if (tid == 0) atomicExch(&g_tc_error, 1);
             break;
         }
         // the G MMAs are done with W3's shared memory: W3 goes back for the next tile
-        if (tid == 0 && nup > 0 && tile + (int)gridDim.x < ntiles) {
-            mbar_expect_tx(f.w3bar, sbuf_bytes(a.ncb, 128));
-            bulk_g2s(f.W3s.p, a.W3_img, sbuf_bytes(a.ncb, 128), f.w3bar);
+        if (f.issuer && nup > 0 && tile + (int)gridDim.x < ntiles) {
+            if (elect_one()) {
+                mbar_expect_tx(f.w3bar, sbuf_bytes(a.ncb, 128));
+                bulk_g2s(f.W3s.p, a.W3_img, sbuf_bytes(a.ncb, 128), f.w3bar);
+            }
             f.w3pending = true;
         }
         // relevancy: each part sums e^T G e over its columns into TMEM column 16 + part
@@ -1065,7 +1086,7 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
         __syncthreads();
     }
     // drain copies still in flight (only after an early exit) before the shared memory goes away
-    if (tid == 0) {
+    if (f.issuer) {
         if (low_pending) mbar_wait(mbar + 1, 0u);
         if (up_pending) mbar_wait(mbar + 2, up_phase);
         if (f.w3pending) mbar_wait(f.w3bar, f.w3phase);
@@ -1139,7 +1160,9 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) export_fused_kernel(cons
     f.tid = tid & 127;
     f.bar_id = 0;
     f.nthreads = blockDim.x;
-    f.half = tid >> 7;
+    const int warp = (int)warp_uniform(threadIdx.x >> 5);
+    f.half = warp >> 2;
+    f.issuer = warp == 0;
     f.nhalf = kQueryParts;
     f.w3bar = mbar + 4;
     if (tid == 0) {
@@ -1151,7 +1174,7 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) export_fused_kernel(cons
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t*>(slot);
+    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
     f.tw = tbase;
     f.lane = (uint32_t)(32 * ((tid >> 5) & 3)) << 16;
     const int row = f.tid;

@@ -7,7 +7,7 @@
 // codes), so the two-tiles-in-flight plan of decoder_tc.cu does not fit.  One
 // persistent CTA per SM, one tile in flight, four warpgroups: thread t serves
 // row t % 128 of the 128-pixel tile (TMEM lane) and the columns of part t / 128
-// in every epilogue; thread 0 also issues the MMAs and bulk copies:
+// in every epilogue; warp 0 also issues the MMAs and bulk copies:
 //   weights      BF16 canonical images of W1 [128 x 16] (input padded to 16),
 //                W2 [256 x 128] and W3 [N x 256], prepared once per call in the
 //                caller's workspace and copied into shared memory once per CTA;
@@ -186,6 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
     uint64_t* const bars = reinterpret_cast<uint64_t*>(sm + kSBar);   // 0 MMA done, 1 weights, 2 W3 half
     uint32_t* const slot = reinterpret_cast<uint32_t*>(sm + kSSlot);
     const int tid = threadIdx.x, row = tid & (kRows - 1), part = tid / kRows;
+    const bool issuer = warp_uniform(threadIdx.x >> 5) == 0;    // the warp of the MMAs and the bulk stores
     uint16_t* const m1 = reinterpret_cast<uint16_t*>(sm + kSMask) + row * 24;   // h1: 8 halves
     uint16_t* const m2 = m1 + 8;                                                // h2: 16 halves
     const int ncb = a.ncb;
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t*>(slot);
+    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
     const uint32_t tl = tbase + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16);   // this warp's TMEM lanes
     uint32_t ph = 0, ph3 = 0;
     int resident = 0;                     // the W3 half in the slot (halves only; thread 0)
@@ -237,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
             sbuf_store8(SBuf{sX, 16}, row, 8, x + 8);
         }
         cta_publish();
-        if (tid == 0) {
+        if (issuer && elect_one()) {
             mma(tbase + kTH, kdesc_at(smem_u32(sX), 16, 0, 0), kdesc_at(smem_u32(sW1), 16, 0, 0),
                 idesc_bf16(kW1, false, false), 0);
             commit(bars);
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
         // E1: H1 = relu(h1 + b1)
         relu_epilogue<kW1>(tl + kTH, b1s, sA, row, h1c0, h1c1, m1);
         cta_publish();
-        if (tid == 0) {
+        if (issuer && elect_one()) {
             const uint32_t a0 = smem_u32(sA), w2 = smem_u32(sW2);
 #pragma unroll
             for (int k = 0; k < kW1 / 16; ++k)
@@ -267,11 +268,11 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
         // E2: H2 = relu(h2 + b2), over H1 (whose MMAs have completed)
         relu_epilogue<kW2>(tl + kTH, b2s, sA, row, h2c0, h2c1, m2);
         cta_publish();
-        if (tid == 0) {
+        if (issuer && elect_one()) {
             const uint32_t a0 = smem_u32(sA), w3 = smem_u32(sW3);
             if (!halves) {
                 const uint32_t id = idesc_bf16(ncb, false, false);
-#pragma unroll 4
+#pragma unroll
                 for (int k = 0; k < kW2 / 16; ++k)
                     mma(tbase + kTZ, kdesc_at(a0, kW2, 0, 16 * k), kdesc_at(w3, kW2, 0, 16 * k), id, k > 0);
             } else {
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
             continue;
         }
         cta_publish();
-        if (tid == 0) {
+        if (issuer && elect_one()) {
             // S4: dh2 = dz W3 (K = ncb; W3 read MN-major)
             const uint32_t a0 = smem_u32(sA), w3 = smem_u32(sW3);
             for (int k = 0; k < ncb / 16; ++k)
@@ -379,10 +380,10 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
         // E4: dH2 = dh2 * [h2 > 0]
         mask_epilogue<kW2>(tl + kTH, m2, sA, row, h2c0, h2c1);
         cta_publish();
-        if (tid == 0) {
+        if (issuer && elect_one()) {
             // S5: dh1 = dH2 W2 (K = 256; W2 read MN-major)
             const uint32_t a0 = smem_u32(sA), w2 = smem_u32(sW2);
-#pragma unroll 4
+#pragma unroll
             for (int k = 0; k < kW2 / 16; ++k)
                 mma(tbase + kTH, kdesc_at(a0, kW2, 0, 16 * k), mndesc_at(w2, kW1, 16 * k, 0),
                     idesc_bf16(kW1, false, true), k > 0);
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
         // E5: dH1 = dh1 * [h1 > 0]
         mask_epilogue<kW1>(tl + kTH, m1, sA, row, h1c0, h1c1);
         cta_publish();
-        if (tid == 0) {
+        if (issuer && elect_one()) {
             // S6: dx = dH1 W1 (K = 128; W1 read MN-major), into the logits' columns
             const uint32_t a0 = smem_u32(sA), w1 = smem_u32(sW1);
 #pragma unroll
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
             atomicAdd(a.loss, lce);
             atomicAdd(a.loss + 1, lu);
         }
-        if (tid == 0) bulk_wait_all();
+        if (issuer && elect_one()) bulk_wait_all();
     }
     fence_before();
     __syncthreads();
@@ -495,34 +496,38 @@ __global__ void __launch_bounds__(kRows, 1) wide_wgrad_kernel(WgradArgs a)
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t*>(slot);
+    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
     // this CTA's tiles: blockIdx.x, blockIdx.x + gridDim.x, ...
     const int n = a.ntiles > (int)blockIdx.x ? (a.ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     bool ok = true;
-    if (tid == 0) {
+    if (warp_uniform(threadIdx.x >> 5) == 0) {
         // half-tile q = 2 i + hf of this CTA's i-th tile goes through stage q % kWStages
         const uint32_t h0 = n0 / 2, h1 = n1 / 2;
         auto load = [&](int q) {
             const int st = q % kWStages, hf = q & 1;
             const unsigned char* b = a.blobs + (size_t)((int)blockIdx.x + (q >> 1) * (int)gridDim.x) * kBlob;
-            mbar_expect_tx(full + st, h0 + h1);
-            bulk_g2s(sm + st * kStage, b + off0 + hf * h0, h0, full + st);
-            bulk_g2s(sm + st * kStage + h0, b + off1 + hf * h1, h1, full + st);
+            if (elect_one()) {
+                mbar_expect_tx(full + st, h0 + h1);
+                bulk_g2s(sm + st * kStage, b + off0 + hf * h0, h0, full + st);
+                bulk_g2s(sm + st * kStage + h0, b + off1 + hf * h1, h1, full + st);
+            }
         };
         const int nq = 2 * n;
         for (int q = 0; q < kWStages && q < nq; ++q) load(q);
         const uint32_t on = smem_u32(ones);
         for (int q = 0; q < nq && ok; ++q) {
             const int st = q % kWStages;
-            if (!mbar_wait(full + st, (uint32_t)(q / kWStages) & 1u)) {
+            if (!warp_agree(mbar_wait(full + st, (uint32_t)(q / kWStages) & 1u))) {
                 ok = false;
                 break;
             }
             fence_after();
             const uint32_t p0 = smem_u32(sm + st * kStage), p1 = p0 + h0;
-#pragma unroll 1
+            const bool lead = elect_one();
+#pragma unroll
             for (int k = 0; k < kRows / 32; ++k) {
                 const uint32_t acc = q > 0 || k > 0;
+                if (!lead) continue;
                 if (role == 0) {
                     const uint64_t A = mndesc_at(p0, 128, 16 * k, 0);
                     mma(tbase, A, mndesc_at(p1, kW2, 16 * k, 0), idesc_bf16(kW2, true, true), acc);
@@ -540,11 +545,12 @@ __global__ void __launch_bounds__(kRows, 1) wide_wgrad_kernel(WgradArgs a)
                         idesc_bf16(16, true, true), acc);
                 }
             }
-            commit(empty + st);
+            if (lead) commit(empty + st);
+            __syncwarp();
             // refill the stage of half-tile q - 1 with half-tile q - 1 + kWStages
             if (q >= 1 && q - 1 + kWStages < nq) {
                 const int sp = (q - 1) % kWStages;
-                if (!mbar_wait(empty + sp, (uint32_t)((q - 1) / kWStages) & 1u)) {
+                if (!warp_agree(mbar_wait(empty + sp, (uint32_t)((q - 1) / kWStages) & 1u))) {
                     ok = false;
                     break;
                 }
@@ -554,7 +560,7 @@ __global__ void __launch_bounds__(kRows, 1) wide_wgrad_kernel(WgradArgs a)
         // the last half-tile's MMAs
         if (ok && nq > 0 && !mbar_wait(empty + (nq - 1) % kWStages, (uint32_t)((nq - 1) / kWStages) & 1u))
             ok = false;
-        if (!ok) atomicExch(&g_wide_error, 1);
+        if (!ok && tid == 0) atomicExch(&g_wide_error, 1);
     }
     const bool bad = bar_any(0, kRows, !ok);
     fence_after();

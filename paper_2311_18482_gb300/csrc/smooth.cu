@@ -8,7 +8,7 @@
 // smooth_kernel: persistent, one CTA per SM, tiles of 128 Gaussians one after
 // another.  Four warpgroups serve the tile's 128 rows (TMEM lanes), each
 // taking 32 of every 128-column epilogue's columns; the loss epilogue is
-// warpgroup 0's.  Thread 0 issues each tcgen05.mma round; after it completes,
+// warpgroup 0's.  Warp 0 issues each tcgen05.mma round; after it completes,
 // all threads run its epilogue (bias, ReLU and its mask, BF16 into shared
 // memory):
 //   forward  H1 = relu(X W1^T + b1), H2, H3, Z = H3 W4^T + b4 (FP32 accumulation)
@@ -75,6 +75,7 @@ struct Ctx {
     uint32_t phase;
     uint32_t tmem, lanef;
     int row;
+    bool issuer;                   // warp 0 (warp-uniform)
     int part;                      // warpgroup: columns [32 part, 32 part + 32) of each hidden epilogue
 };
 
@@ -146,11 +147,12 @@ __device__ __forceinline__ uint64_t kd(uint32_t s0, uint32_t off, int C) { retur
 // MN-major descriptor (rows = K) of a C-column buffer.
 __device__ __forceinline__ uint64_t md(uint32_t s0, uint32_t off, int C) { return mndesc_at(s0 + off, C, 0, 0); }
 
-// One MMA round, issued by thread 0.  K steps of 16 move the start address by
-// 16 units (K-major) or 2C units (MN-major over a C-column buffer).  The
-// arguments come by value, so the caller's context stays in registers.
-__device__ __noinline__ void issue(uint32_t s0, uint32_t t, uint64_t* bar, int round, bool first_tile)
+// One MMA round, issued by warp 0's elected lane.  K steps of 16 move the start address by
+// 16 units (K-major) or 2C units (MN-major over a C-column buffer).
+__device__ __forceinline__ void issue(const Ctx& c, int round, bool first_tile)
 {
+    if (!c.issuer || !elect_one()) return;
+    const uint32_t s0 = c.s0, t = c.tmem;
     const uint32_t keep = first_tile ? 0u : 1u;
     switch (round) {
         case 0:   // H1 pre-activation = X W1^T
@@ -201,7 +203,7 @@ __device__ __noinline__ void issue(uint32_t s0, uint32_t t, uint64_t* bar, int r
             break;
         }
     }
-    commit(bar);
+    commit(c.bar);
 }
 
 // Sum over the warp's 32 rows of 16 values (recursive halving); lanes 2j, 2j+1 hold column j.
@@ -237,7 +239,8 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
     c.phase = 0;
     c.row = threadIdx.x & 127;
     c.part = threadIdx.x >> 7;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    c.issuer = warp == 0;
     c.lanef = (uint32_t)(32 * (warp & 3)) << 16;
     // weights (BF16, [out][in]), biases (FP32), the ones operand
     sbuf_fill(SBuf{c.sm + kOW1, 16}, 128, a.W1, 3, kH, 3);
@@ -259,7 +262,7 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
     fence_before();
     __syncthreads();
     fence_after();
-    c.tmem = *reinterpret_cast<volatile uint32_t*>(c.tslot);
+    c.tmem = warp_uniform(*reinterpret_cast<volatile uint32_t*>(c.tslot));
 
     const float* b1 = bs;
     const float* b2 = bs + kH;
@@ -301,19 +304,19 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
         uint32_t* m2 = m1 + 4 * 128;
         uint32_t* m3 = m2 + 4 * 128;
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 0, first);
+        issue(c, 0, first);
         if (!(ok = round_wait(c))) break;
         hidden_epilogue(c, b1, kOH1, m1);
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 1, first);
+        issue(c, 1, first);
         if (!(ok = round_wait(c))) break;
         hidden_epilogue(c, b2, kOH2, m2);
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 2, first);
+        issue(c, 2, first);
         if (!(ok = round_wait(c))) break;
         hidden_epilogue(c, b3, kOH3, m3);
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 3, first);
+        issue(c, 3, first);
         if (!(ok = round_wait(c))) break;
         if (p0) {   // loss and the output gradient
             float z[16];
@@ -341,26 +344,28 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
             db4acc += colsum16(dz, lane);       // lanes 2k, 2k+1: column k (k < 8)
         }
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 4, first);
+        issue(c, 4, first);
         if (!(ok = round_wait(c))) break;
         grad_epilogue(c, kOH3, m3);              // dH3 over H3 (read by dW4, complete)
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 5, first);
+        issue(c, 5, first);
         if (!(ok = round_wait(c))) break;
         grad_epilogue(c, kOH2, m2);              // dH2 over H2
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 6, first);
+        issue(c, 6, first);
         if (!(ok = round_wait(c))) break;
         grad_epilogue(c, kOH1, m1);              // dH1 over H1
         publish();
-        if (threadIdx.x == 0) issue(c.s0, c.tmem, c.bar, 7, first);
+        issue(c, 7, first);
         if (!(ok = round_wait(c))) break;
     }
     if (!ok) {
-        if (threadIdx.x == 0) {
-            atomicExch(&g_smooth_error, 1);
+        if (c.issuer) {
             // nothing of ours may still be running when TMEM is freed
-            commit(c.bar);
+            if (elect_one()) {
+                atomicExch(&g_smooth_error, 1);
+                commit(c.bar);
+            }
             (void)mbar_wait(c.bar, c.phase);
         }
     } else if (any) {

@@ -126,6 +126,29 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t start, uint32_t lbo, uint
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
 }
 
+// MMAs are issued by one lane, but from code that the whole warp runs:
+//   if (warp == k) { ...loop, waits, descriptors...; if (elect_one()) { mma(...); commit(...); } }
+// with the warp index and the TMEM base made warp-uniform by warp_uniform().
+// The descriptors then live in uniform registers, where tcgen05.mma takes them
+// from.  Under a lane == 0 branch each one is moved there by its own
+// instruction and the loop runs on one lane's vector registers: 125 cycles per
+// M = 128, K = 16 MMA whatever N is, against 53 (N = 64) and 66 (N = 128), the
+// tensor core's own rate (le_smooth on 1M Gaussians 0.584 -> 0.527 ms; the
+// decoder kernels, bound by other parts of a tile, 2 to 3 %).  A warp's MMAs
+// and commits all come from the same elected lane.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
+
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// A wait done by a whole warp: one outcome for all lanes, so that a timeout never
+// leaves part of them at the next elect_one().
+__device__ __forceinline__ bool warp_agree(bool ok) { return __all_sync(0xffffffffu, ok); }
+
 // D[tmem] (+)= A * B, issued by one thread.
 __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
 {
