@@ -94,6 +94,20 @@ struct Front {
     bool w3pending = false;
 };
 
+__device__ __forceinline__ float4 ld_bias4(const float* b, int c) { return *reinterpret_cast<const float4*>(b + c); }
+
+__device__ __forceinline__ void add_bias16(float* v, const float* b, int c)
+{
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) {
+        const float4 bb = ld_bias4(b, c + j);
+        v[j] += bb.x;
+        v[j + 1] += bb.y;
+        v[j + 2] += bb.z;
+        v[j + 3] += bb.w;
+    }
+}
+
 // Columns [c0, c1) of an N-column epilogue handled by this thread's half (units of 16).
 __device__ __forceinline__ void my_cols(const Front& f, int N, int& c0, int& c1)
 {
@@ -129,9 +143,6 @@ __device__ __forceinline__ void wg_publish(const Front& f)
     fence_after();
 }
 
-// D_MLP forward of one 128-pixel tile: X1 <- feat (col 8 = 1 for the bias
-// gradient), H1 = relu(W1 x + b1), H2 = relu(W2 h1 + b2), logits - b3 left in
-// TMEM columns [tw, tw + ncb).  Returns false on a timed-out wait.
 // R_s of pixel p (zeros past the end), for mlp_forward_x.
 __device__ __forceinline__ void load_feat(const DecArgs& a, int p, bool valid, float* x)
 {
@@ -139,8 +150,11 @@ __device__ __forceinline__ void load_feat(const DecArgs& a, int p, bool valid, f
     for (int c = 0; c < 8; ++c) x[c] = valid ? a.feat[(size_t)c * a.P + p] : 0.f;
 }
 
-// mlp_forward with the tile's features already in registers (x, read by the
-// first part only), so that a caller can load them a tile ahead.
+// D_MLP forward of one 128-pixel tile: X1 <- x (col 8 = 1 for the bias
+// gradient), H1 = relu(W1 x + b1), H2 = relu(W2 h1 + b2), logits - b3 left in
+// TMEM columns [tw, tw + ncb).  The tile's features come in registers (x, read
+// by the first part only), so that a caller can load them a tile ahead.
+// Returns false on a timed-out wait.
 __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
 {
     float v[16];
@@ -160,8 +174,9 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
     my_cols(f, kH1, c0, c1);
     for (int c = c0; c < c1; c += 16) {
         tmem_ld16(f.tw + f.lane + c, v);
+        add_bias16(v, f.b1s, c);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j] + f.b1s[c + j], 0.f);
+        for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j], 0.f);
         sbuf_store8(f.H1, f.tid, c, v);
         sbuf_store8(f.H1, f.tid, c + 8, v + 8);
     }
@@ -176,8 +191,9 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
     my_cols(f, kH2, c0, c1);
     for (int c = c0; c < c1; c += 16) {
         tmem_ld16(f.tw + f.lane + c, v);
+        add_bias16(v, f.b2s, c);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j] + f.b2s[c + j], 0.f);
+        for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j], 0.f);
         sbuf_store8(f.H2, f.tid, c, v);
         sbuf_store8(f.H2, f.tid, c + 8, v + 8);
     }
@@ -199,57 +215,25 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
     return wg_wait(f);
 }
 
-__device__ bool mlp_forward(Front& f, const DecArgs& a, int p, bool valid)
-{
-    float x[8];
-    if (f.half == 0) load_feat(a, p, valid, x);
-    return mlp_forward_x(f, a, x);
-}
-
-// Online max / argmax / log-sum-exp over the ncb logits in TMEM (+ b3); with
-// several parts, each covers its columns and they combine through f.xch in
-// column order.  Ties go to the lowest index.  zt = logit of class t (if t >= 0).
-__device__ __forceinline__ void logits_lse(const Front& f, int ncb, float& lse, int& am, int t, float& zt)
+// Online max / argmax / log-sum-exp over the ncb logits in TMEM (+ b3), ties to
+// the lowest index.  Without a branch per column: a new maximum (s e + 1) and a
+// smaller logit (s 1 + e) are one FMA of selected factors, e = exp(-|z - max|).
+__device__ __forceinline__ void logits_lse(const Front& f, int ncb, float& lse, int& am)
 {
     float m = -INFINITY, s = 0.f, v[16];
     am = 0;
-    zt = 0.f;
-    int c0, c1;
-    my_cols(f, ncb, c0, c1);
-    for (int c = c0; c < c1; c += 16) {
+    for (int c = 0; c < ncb; c += 16) {
         tmem_ld16(f.tw + f.lane + c, v);
+        add_bias16(v, f.b3s, c);
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-            const float z = v[j] + f.b3s[c + j];
-            if (c + j == t) zt = z;
-            if (z > m) {
-                s = s * __expf(m - z) + 1.f;
-                m = z;
-                am = c + j;
-            } else {
-                s += __expf(z - m);
-            }
+            const float z = v[j];
+            const bool up = z > m;
+            const float e = __expf(-fabsf(z - m));
+            s = __fmaf_rn(s, up ? e : 1.f, up ? 1.f : e);
+            m = up ? z : m;
+            am = up ? c + j : am;
         }
-    }
-    if (f.nhalf > 1) {
-        f.xch[f.half * 128 + f.tid] = make_float4(m, s, __int_as_float(am), zt);
-        wg_sync(f);
-        float mt = -INFINITY, st = 0.f, zsum = 0.f;
-        int at = 0;
-        for (int h = 0; h < f.nhalf; ++h) {
-            const float4 o = f.xch[h * 128 + f.tid];
-            if (o.x == -INFINITY) continue;           // a part without columns
-            const float mn = fmaxf(mt, o.x);
-            st = (mt == -INFINITY ? 0.f : st * __expf(mt - mn)) + o.y * __expf(o.x - mn);
-            if (o.x > mt) at = __float_as_int(o.z);
-            mt = mn;
-            zsum += o.w;                             // only the part holding class t has it
-        }
-        wg_sync(f);
-        m = mt;
-        s = st;
-        am = at;
-        zt = zsum;
     }
     lse = m + __logf(s);
 }
@@ -273,8 +257,8 @@ __device__ unsigned char* load_weights(unsigned char* base, const DecArgs& a, Fr
     float* bs = reinterpret_cast<float*>(p);
     p += ((size_t)(64 + 128 + a.ncb) * 4 + 127) / 128 * 128;
     sbuf_fill(f.W1s, 64, a.W1, kD, 64, kD);
-    sbuf_fill(f.W2s, 128, a.W2, kH1, 128, kH1);
-    sbuf_fill(f.W3s, a.ncb, a.W3, kH2, a.ncb, kH2);
+    sbuf_fill_rows(f.W2s, 128, a.W2);
+    sbuf_fill_rows(f.W3s, a.ncb, a.W3);
     for (int i = threadIdx.x; i < 64 + 128 + a.ncb; i += blockDim.x)
         bs[i] = i < 64 ? a.b1[i] : (i < 192 ? a.b2[i - 64] : a.b3[i - 192]);
     f.b1s = bs;
@@ -284,24 +268,33 @@ __device__ unsigned char* load_weights(unsigned char* base, const DecArgs& a, Fr
 }
 
 // ---------------------------------------------------------------------------
-// Inference.  NWG warpgroups per CTA, each with its own tile, buffers,
-// mbarrier and 256 TMEM columns; weights shared.
+// Inference.  NWG warpgroups per CTA, each with its own tile, buffers, mbarrier
+// and 512 / NWG TMEM columns; weights shared.  A tile is a chain of three MMA
+// rounds and their epilogues, so the tiles in flight per SM set the rate: four
+// up to 128 codes (H2 takes the place of X1 and H1, which have been read by
+// then), two above, where a tile's logits need 256 columns.  Tiles are dealt out
+// over the CTAs first, so a small image spreads over the SMs.  With two tiles of
+// 128 codes in flight and a branch per logit in the softmax, 10,000 / 300,000 /
+// 1,088,640 pixels took 19.8 / 114 / 370 us at 128 codes and 31.8 / 194 / 629 us
+// at 256; now 10.3 / 52 / 157 us and 14.7 / 100 / 322 us.
 constexpr size_t kFwdWgBytes = sbuf_bytes(128, 16) + sbuf_bytes(128, 64) + sbuf_bytes(128, 128);
+constexpr size_t kFwdTileBytes = sbuf_bytes(128, 128);
 
-__host__ constexpr size_t fwd_smem(int ncb, int nwg) { return weights_bytes(ncb) + nwg * kFwdWgBytes + 128; }
+__host__ constexpr size_t fwd_smem(int ncb, int nwg) { return weights_bytes(ncb) + nwg * kFwdTileBytes + 128; }
 
 template <int NWG>
 __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
+    constexpr int kCols = 512 / NWG;
     Front f;
     unsigned char* p = load_weights(sm, a, f);
     const int warp = (int)warp_uniform(threadIdx.x >> 5), wg = warp >> 2;
-    unsigned char* q = p + wg * kFwdWgBytes;
+    unsigned char* q = p + wg * kFwdTileBytes;
     f.X1 = SBuf{q, 16};
     f.H1 = SBuf{q + sbuf_bytes(128, 16), 64};
-    f.H2 = SBuf{q + sbuf_bytes(128, 16) + sbuf_bytes(128, 64), 128};
-    uint64_t* mbars = reinterpret_cast<uint64_t*>(p + NWG * kFwdWgBytes);
+    f.H2 = SBuf{q, 128};
+    uint64_t* mbars = reinterpret_cast<uint64_t*>(p + NWG * kFwdTileBytes);
     uint32_t* slot = reinterpret_cast<uint32_t*>(mbars + NWG);
     f.mbar = mbars + wg;
     f.phase = 0;
@@ -314,31 +307,38 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
     f.xch = nullptr;
     if (threadIdx.x == 0)
         for (int w = 0; w < NWG; ++w) mbar_init(mbars + w, 1);
-    if (threadIdx.x < 32) tmem_alloc(slot, 256 * NWG);
+    if (threadIdx.x < 32) tmem_alloc(slot, 512);
     fence_proxy_async();
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
-    f.tw = tbase + 256 * wg;
+    f.tw = tbase + kCols * wg;
     f.lane = (uint32_t)(32 * (f.tid >> 5)) << 16;
 
     const int ntiles = (a.P + 127) / 128;
-    for (int tile = blockIdx.x * NWG + wg; tile < ntiles; tile += gridDim.x * NWG) {
+    const auto tile_px = [&](int tile) { return tile < ntiles ? tile * 128 + f.tid : a.P; };
+    float x[8];                                 // this tile's R_s, loaded a tile ahead
+    int tile = blockIdx.x + gridDim.x * wg;
+    load_feat(a, tile_px(tile), tile_px(tile) < a.P, x);
+    for (; tile < ntiles; tile += gridDim.x * NWG) {
         const int px = tile * 128 + f.tid;
         const bool valid = px < a.P;
-        if (!mlp_forward(f, a, px, valid)) break;
-        float lse, zt;
+        if (!mlp_forward_x(f, a, x)) break;
+        const int nx = tile_px(tile + (int)gridDim.x * NWG);
+        load_feat(a, nx, nx < a.P, x);
+        float lse;
         int am;
-        logits_lse(f, a.ncb, lse, am, -1, zt);
+        logits_lse(f, a.ncb, lse, am);
         if (valid && a.argmax) a.argmax[px] = am;
         if (a.prob) {
             float v[16];
             for (int c = 0; c < a.ncb; c += 16) {
                 tmem_ld16(f.tw + f.lane + c, v);
+                add_bias16(v, f.b3s, c);
                 if (valid)
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) a.prob[(size_t)(c + j) * a.P + px] = __expf(v[j] + f.b3s[c + j] - lse);
+                    for (int j = 0; j < 16; ++j) a.prob[(size_t)(c + j) * a.P + px] = __expf(v[j] - lse);
             }
         }
         fence_before();
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
     fence_before();
     __syncthreads();
     fence_after();
-    if (threadIdx.x < 32) tmem_dealloc(tbase, 256 * NWG);
+    if (threadIdx.x < 32) tmem_dealloc(tbase, 512);
 }
 
 // ---------------------------------------------------------------------------
@@ -518,8 +518,6 @@ __device__ __forceinline__ uint32_t xch_off(int i)
     return (uint32_t)((i >> 4) * 2048 + ((i >> 3) & 1) * 128 + (i & 7) * 16);
 }
 
-__device__ __forceinline__ float4 ld_bias4(const float* b, int c) { return *reinterpret_cast<const float4*>(b + c); }
-
 // bias + ReLU over 16 columns starting at c: v <- relu(v + b); bit j of the
 // result = (v_j > 0)
 __device__ __forceinline__ uint32_t bias_relu16(float* v, const float* b, int c)
@@ -565,18 +563,6 @@ __device__ __forceinline__ float select16(const float* v, int idx)
 #pragma unroll
     for (int i = 0; i < 2; ++i) t2[i] = b2 ? t4[2 * i + 1] : t4[2 * i];
     return b3 ? t2[1] : t2[0];
-}
-
-__device__ __forceinline__ void add_bias16(float* v, const float* b, int c)
-{
-#pragma unroll
-    for (int j = 0; j < 16; j += 4) {
-        const float4 bb = ld_bias4(b, c + j);
-        v[j] += bb.x;
-        v[j + 1] += bb.y;
-        v[j + 2] += bb.z;
-        v[j + 3] += bb.w;
-    }
 }
 
 __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bias, EpiCtx& e, int ntiles,
@@ -1474,12 +1460,13 @@ le_status decode_fused(int32_t P, const float* feat, const float* unc, const le_
         LE_LAUNCHED();
         return LE_OK;
     }
-    const size_t smem = fwd_smem(a.ncb, 2);
-    le_status st = set_smem(dec_fwd_kernel<2>, smem);
+    const int nwg = a.ncb <= 128 ? 4 : 2, sms = sm_count();
+    const size_t smem = fwd_smem(a.ncb, nwg);
+    le_status st = nwg == 4 ? set_smem(dec_fwd_kernel<4>, smem) : set_smem(dec_fwd_kernel<2>, smem);
     if (st != LE_OK) return st;
-    const int want = (ntiles + 1) / 2;
-    const int grid = want < sm_count() ? want : sm_count();
-    dec_fwd_kernel<2><<<grid, 256, smem, s>>>(a);
+    const int grid = ntiles < sms ? ntiles : sms;
+    if (nwg == 4) dec_fwd_kernel<4><<<grid, 512, smem, s>>>(a);
+    else dec_fwd_kernel<2><<<grid, 256, smem, s>>>(a);
     LE_LAUNCHED();
     return LE_OK;
 }

@@ -83,15 +83,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
                  : "memory");
 }
 
-// 1-D bulk copy this CTA's shared memory -> global, counted in this thread's
-// bulk async-group (16-byte aligned addresses, size a multiple of 16).
-__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
-                 "r"(bytes)
-                 : "memory");
-}
-
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 
 // Until this thread's committed bulk stores have read their shared-memory source.
@@ -302,6 +293,34 @@ __device__ __forceinline__ void sbuf_fill(const SBuf& b, int R, const float* src
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = (r < rs && c0 + j < cs) ? src[(size_t)r * ld + c0 + j] : 0.f;
         sbuf_store8(b, r, c0, v);
+    }
+}
+
+// The same for a whole [R x C] matrix at a 16-byte aligned address, four 8-column
+// pieces in flight per thread (a kernel's first microseconds are these loads).
+__device__ __forceinline__ void sbuf_fill_rows(const SBuf& b, int R, const float* src)
+{
+    if (reinterpret_cast<uintptr_t>(src) & 15u) {
+        sbuf_fill(b, R, src, b.C, R, b.C);
+        return;
+    }
+    const int w = b.C >> 3, pieces = R * w;
+    const float4* s4 = reinterpret_cast<const float4*>(src);
+    for (int i0 = threadIdx.x; i0 < pieces; i0 += 4 * blockDim.x) {
+        float4 x[4][2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = i0 + q * blockDim.x;
+            if (i < pieces) {
+                x[q][0] = __ldg(s4 + 2 * i);
+                x[q][1] = __ldg(s4 + 2 * i + 1);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = i0 + q * blockDim.x;
+            if (i < pieces) sbuf_store8(b, i / w, (i % w) * 8, reinterpret_cast<const float*>(x[q]));
+        }
     }
 }
 

@@ -108,6 +108,24 @@ def test_fused_inference(leg, orc, P, ncb):
     assert dp <= 1e-2
 
 
+@pytest.mark.parametrize("P,ncb", [(127, 128), (129, 112), (77824 + 130, 128), (127, 144), (38912 + 130, 144)])
+def test_fused_inference_tiles(leg, P, ncb):
+    """Four tiles in flight per CTA up to 128 codes and two above, one to several tiles per warpgroup:
+    probabilities within 2e-3 of the BF16 emulation, its argmax wherever the top two logits are 1e-3 apart."""
+    import paper_2311_18482_gb300 as L
+    dec = synth.decoder_init(41, ncb)
+    feat, _, _ = _inputs(P, ncb, 42)
+    out = L.le_decode(L.FUSED_BF16, _t(feat), _dec_t(dec), want_prob=True)
+    L.le_device_status()
+    ze = emulate_logits(feat, dec)
+    zs = np.sort(ze, axis=0)
+    clear = (zs[-1] - zs[-2]) > 1e-3
+    pe = np.exp(ze - ze.max(0))
+    pe /= pe.sum(0)
+    assert np.array_equal(to_np(out["argmax"])[clear], np.argmax(ze, 0)[clear])
+    assert np.max(np.abs(to_np(out["prob"]) - pe)) <= 2e-3
+
+
 @pytest.mark.parametrize("P,ncb", [(3001, 128), (20000, 64), (1500, 16)])
 def test_fused_train(leg, orc, P, ncb):
     import paper_2311_18482_gb300 as L
