@@ -94,20 +94,6 @@ struct Front {
     bool w3pending = false;
 };
 
-__device__ __forceinline__ float4 ld_bias4(const float* b, int c) { return *reinterpret_cast<const float4*>(b + c); }
-
-__device__ __forceinline__ void add_bias16(float* v, const float* b, int c)
-{
-#pragma unroll
-    for (int j = 0; j < 16; j += 4) {
-        const float4 bb = ld_bias4(b, c + j);
-        v[j] += bb.x;
-        v[j + 1] += bb.y;
-        v[j + 2] += bb.z;
-        v[j + 3] += bb.w;
-    }
-}
-
 // Columns [c0, c1) of an N-column epilogue handled by this thread's half (units of 16).
 __device__ __forceinline__ void my_cols(const Front& f, int N, int& c0, int& c1)
 {
@@ -158,6 +144,7 @@ __device__ __forceinline__ void load_feat(const DecArgs& a, int p, bool valid, f
 __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
 {
     float v[16];
+    uint32_t w[8];
     if (f.half == 0) sbuf_store8(f.X1, f.tid, 0, x);
     if (f.half == f.nhalf - 1) {
 #pragma unroll
@@ -174,11 +161,8 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
     my_cols(f, kH1, c0, c1);
     for (int c = c0; c < c1; c += 16) {
         tmem_ld16(f.tw + f.lane + c, v);
-        add_bias16(v, f.b1s, c);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j], 0.f);
-        sbuf_store8(f.H1, f.tid, c, v);
-        sbuf_store8(f.H1, f.tid, c + 8, v + 8);
+        relu16(v, f.b1s + c, w);
+        sts_row16(smem_u32(f.H1.p) + sbuf_off(f.tid, c, f.H1.C), w);
     }
     wg_publish(f);
     if (f.issuer && elect_one()) {
@@ -191,11 +175,8 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
     my_cols(f, kH2, c0, c1);
     for (int c = c0; c < c1; c += 16) {
         tmem_ld16(f.tw + f.lane + c, v);
-        add_bias16(v, f.b2s, c);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j], 0.f);
-        sbuf_store8(f.H2, f.tid, c, v);
-        sbuf_store8(f.H2, f.tid, c + 8, v + 8);
+        relu16(v, f.b2s + c, w);
+        sts_row16(smem_u32(f.H2.p) + sbuf_off(f.tid, c, f.H2.C), w);
     }
     wg_publish(f);
     if (f.issuer) {
@@ -224,7 +205,7 @@ __device__ __forceinline__ void logits_lse(const Front& f, int ncb, float& lse, 
     am = 0;
     for (int c = 0; c < ncb; c += 16) {
         tmem_ld16(f.tw + f.lane + c, v);
-        add_bias16(v, f.b3s, c);
+        add_bias16(v, f.b3s + c);
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             const float z = v[j];
@@ -335,7 +316,7 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
             float v[16];
             for (int c = 0; c < a.ncb; c += 16) {
                 tmem_ld16(f.tw + f.lane + c, v);
-                add_bias16(v, f.b3s, c);
+                add_bias16(v, f.b3s + c);
                 if (valid)
 #pragma unroll
                     for (int j = 0; j < 16; ++j) a.prob[(size_t)(c + j) * a.P + px] = __expf(v[j] - lse);
@@ -356,11 +337,11 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
 // every epilogue by columns), so the tensor core works on one slot while the
 // CUDA cores finish the other.  Per tile, six MMA stages alternate with six
 // epilogues (z = logits, dz = dL/dz etc.):
-//   S1  h1 = X1 W1^T                                E1  bias, ReLU -> H1; ReLU mask kept in registers
-//   S2  h2 = H1 W2^T                                E2  bias, ReLU -> H2; mask
+//   S1  h1 = X1 W1^T                                E1  bias, ReLU -> H1
+//   S2  h2 = H1 W2^T                                E2  bias, ReLU -> H2
 //   S3  z  = H2 W3^T                                E3  softmax, CE (Eqs. 9-12) -> dz into D
-//   S4  dh2 = dz W3;  dW3 += dz^T h2;  db3 += dz^T 1   E4  mask -> dh2 into H2's buffer
-//   S5  dh1 = dh2 W2; dW2 += dh2^T h1; db2 += dh2^T 1  E5  mask -> dh1 into D
+//   S4  dh2 = dz W3;  dW3 += dz^T h2;  db3 += dz^T 1   E4  mask (h2 > 0) -> dh2 into H2's buffer
+//   S5  dh1 = dh2 W2; dW2 += dh2^T h1; db2 += dh2^T 1  E5  mask (h1 > 0) -> dh1 into D
 //   S6  dx  = dh1 W1; [dW1 | db1] += dh1^T [x | 1]     E6  dx -> d_feat
 // dz, dh2 and dh1 are stored pixel-major: the input-gradient MMAs read them
 // K-major and the weight-gradient MMAs MN-major (contracting over the tile's
@@ -518,31 +499,6 @@ __device__ __forceinline__ uint32_t xch_off(int i)
     return (uint32_t)((i >> 4) * 2048 + ((i >> 3) & 1) * 128 + (i & 7) * 16);
 }
 
-// bias + ReLU over 16 columns starting at c: v <- relu(v + b); bit j of the
-// result = (v_j > 0)
-__device__ __forceinline__ uint32_t bias_relu16(float* v, const float* b, int c)
-{
-    uint32_t m = 0;
-#pragma unroll
-    for (int j = 0; j < 16; j += 4) {
-        const float4 bb = ld_bias4(b, c + j);
-        const float bj[4] = {bb.x, bb.y, bb.z, bb.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float x = v[j + i] + bj[i];
-            m |= (x > 0.f ? 1u : 0u) << (j + i);
-            v[j + i] = fmaxf(x, 0.f);
-        }
-    }
-    return m;
-}
-
-__device__ __forceinline__ void mask16(float* v, uint32_t m)
-{
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = (m >> j) & 1u ? v[j] : 0.f;
-}
-
 // 16 columns [c, c + 16) of row `row` of the C-column buffer at shared address b.
 __device__ __forceinline__ void store16(uint32_t b, int C, int row, int c, const float* v)
 {
@@ -628,25 +584,22 @@ __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bi
         fetch(tile + 2 * (int)gridDim.x);
         epi_signal(e);
         if (!epi_wait(e)) return false;
-        // E1: h1 columns [32h, 32h + 32), bits of the ReLU mask in m1
-        uint32_t m1 = 0;
+        // E1: h1 columns [32h, 32h + 32)
+        uint32_t w[8];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             tmem_ld16(tl + 32 * h + 16 * k, v);
-            m1 |= bias_relu16(v, b1s, 32 * h + 16 * k) << (16 * k);
-            store16(H1, kH1, row, 32 * h + 16 * k, v);
+            relu16(v, b1s + 32 * h + 16 * k, w);
+            sts_row16(H1 + sbuf_off(row, 32 * h + 16 * k, kH1), w);
         }
         epi_signal(e);
         if (!epi_wait(e)) return false;
-        // E2: h2 columns [64h, 64h + 64), mask bits in m2a (first 32) and m2b
-        uint32_t m2a = 0, m2b = 0;
+        // E2: h2 columns [64h, 64h + 64)
 #pragma unroll 1
         for (int k = 0; k < 4; ++k) {
             tmem_ld16(tl + 64 * h + 16 * k, v);
-            const uint32_t mk = bias_relu16(v, b2s, 64 * h + 16 * k);
-            if (k < 2) m2a |= mk << (16 * k);
-            else m2b |= mk << (16 * (k - 2));
-            store16(H2, 128, row, 64 * h + 16 * k, v);
+            relu16(v, b2s + 64 * h + 16 * k, w);
+            sts_row16(H2 + sbuf_off(row, 64 * h + 16 * k, 128), w);
         }
         epi_signal(e);
         if (!epi_wait(e)) return false;
@@ -660,7 +613,7 @@ __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bi
         for (int uu = 0; uu < 4; ++uu)
             if (c0 + 16 * uu < c1) {
                 tmem_ld16(tl + c0 + 16 * uu, v);
-                add_bias16(v, b3s, c0 + 16 * uu);
+                add_bias16(v, b3s + c0 + 16 * uu);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) mh = fmaxf(mh, v[j]);
                 if (own_t && (jt >> 4) == uu) zt_h = select16(v, jt & 15);
@@ -671,7 +624,7 @@ __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bi
         for (int uu = 0; uu < 4; ++uu)
             if (c0 + 16 * uu < c1) {
                 tmem_ld16(tl + c0 + 16 * uu, v);
-                add_bias16(v, b3s, c0 + 16 * uu);
+                add_bias16(v, b3s + c0 + 16 * uu);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     v[j] = ex2_approx(fmaf(v[j], kL2E, -mhl));
@@ -699,14 +652,14 @@ __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bi
         const float lse = m + __logf(ssum);
         const float zt = own_t ? zt_h : o.z;
         const float ce = lse - zt;
-        const float w = valid ? a.lambda_ce * (1.f - u) : 0.f;
+        const float wce = valid ? a.lambda_ce * (1.f - u) : 0.f;
         if (valid && h == 0) {
             a.d_unc[px] = (a.lambda_u - a.lambda_ce * ce) * a.invP;
             acc_ce += ce * (1.f - u);
             acc_u += u;
         }
         // dz * P (1/P is applied when the gradients are written)
-        const float scale = c0 < c1 ? w * ex2_approx((mh - m) * kL2E) / ssum : 0.f;
+        const float scale = c0 < c1 ? wce * ex2_approx((mh - m) * kL2E) / ssum : 0.f;
 #pragma unroll 1
         for (int uu = 0; uu < 4; ++uu)
             if (c0 + 16 * uu < c1) {
@@ -717,7 +670,7 @@ __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bi
             }
         if (own_t && valid) {
             const float et = ex2_approx(fmaf(zt_h, kL2E, -mhl));
-            const __nv_bfloat16 bv = __float2bfloat16_rn(et * scale - w);
+            const __nv_bfloat16 bv = __float2bfloat16_rn(et * scale - wce);
             asm volatile("st.shared.b16 [%0], %1;" ::"r"(D + sbuf_off(row, t, 128)),
                          "h"(*reinterpret_cast<const unsigned short*>(&bv))
                          : "memory");
@@ -728,8 +681,9 @@ __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bi
 #pragma unroll 1
         for (int k = 0; k < 4; ++k) {
             tmem_ld16(tl + 64 * h + 16 * k, v);
-            mask16(v, (k < 2 ? m2a : m2b) >> (16 * (k & 1)));
-            store16(H2, 128, row, 64 * h + 16 * k, v);
+            const uint32_t at = H2 + sbuf_off(row, 64 * h + 16 * k, 128);
+            relu_mask16(v, at, w);
+            sts_row16(at, w);
         }
         epi_signal(e);
         if (!epi_wait(e)) return false;
@@ -737,8 +691,8 @@ __device__ __forceinline__ bool train_epilogue(const DecArgs& a, const float* bi
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             tmem_ld16(tl + 32 * h + 16 * k, v);
-            mask16(v, m1 >> (16 * k));
-            store16(D, 128, row, 32 * h + 16 * k, v);
+            relu_mask16(v, H1 + sbuf_off(row, 32 * h + 16 * k, kH1), w);
+            sts_row16(D + sbuf_off(row, 32 * h + 16 * k, 128), w);
         }
         epi_signal(e);
         if (!epi_wait(e)) return false;

@@ -17,8 +17,8 @@
 //   activations  one 64 KB region holds the operand of the next MMA stage --
 //                H1, H2 and, training, dZ, dH2, dH1 -- each written by the
 //                epilogue once the MMAs reading its predecessor have completed;
-//                the ReLU masks of h1 and h2 are kept as bits (4 + 8 words per
-//                row, in shared memory so that the epilogue loops stay rolled).
+//                the ReLU masks of h1 and h2 are kept as bits (8 + 16 words
+//                per row, in shared memory so that the epilogue loops stay rolled).
 //   TMEM         512 columns: [0, 256) hidden-layer accumulators (h1, h2, dh2,
 //                dh1), [256, 256 + N) the logits, later [256, 272) dx.
 // Training (N <= 128) takes two passes:
@@ -37,7 +37,7 @@
 //           by output (dW3 | dW2 | dW1), accumulated in TMEM and added to the
 //           outputs with atomics once per CTA.  Bias gradients are MMAs against
 //           a ones operand (b3, b2) or the ones column 8 of X (b1).
-// A training call on 1,088,640 pixels and 128 codes takes 1.05 ms (1.35 ms with the
+// A training call on 1,088,640 pixels and 128 codes takes 1.00 ms (1.35 ms with the
 // bulk copies, a branch per logit in the softmax and the tile's inputs loaded on
 // its path); the floor of the two passes' own traffic is 0.58 ms.  Inference on
 // the same pixels: 0.317 ms (0.522 ms).
@@ -62,7 +62,7 @@ constexpr uint32_t kW1Bytes = sbuf_bytes(kW1, 16), kW2Bytes = sbuf_bytes(kW2, kW
 // Shared memory of wide_kernel (offsets from a 1024-byte aligned base).
 constexpr uint32_t kSW1 = 0, kSW2 = kSW1 + kW1Bytes, kSW3 = kSW2 + kW2Bytes, kSX = kSW3 + kW3Half,
                    kSA = kSX + kXBytes, kSBias = kSA + kABytes, kSMask = kSBias + (kW1 + kW2 + 256) * 4,
-                   kSXch = kSMask + kRows * 12 * 4, kSBar = kSXch + 4 * kRows * 16, kSSlot = kSBar + 4 * 8,
+                   kSXch = kSMask + kRows * 24 * 4, kSBar = kSXch + 4 * kRows * 16, kSSlot = kSBar + 4 * 8,
                    kSmem = kSSlot + 16;
 
 // One tile's operand images in the training workspace (pass 1 writes, pass 2 reads).
@@ -110,78 +110,60 @@ __device__ __forceinline__ bool wide_wait(uint64_t* bar, uint32_t& phase)
     return !bad;
 }
 
-// 16 columns [c, c + 16) of a row, as BF16, into the canonical C-column buffer
-// and (training) into the tile's copy of it in the workspace: eight rows' 16-byte
-// units are consecutive, so a warp's store covers whole 128-byte lines.
+// 16 columns [c, c + 16) of a row (eight BF16 pairs) into the canonical C-column
+// buffer and (training) into the tile's copy of it in the workspace: eight rows'
+// 16-byte units are consecutive, so a warp's store covers whole 128-byte lines.
 template <bool TRAIN, int C>
-__device__ __forceinline__ void store_cols(unsigned char* dst, unsigned char* image, int row, int c, const float* v)
+__device__ __forceinline__ void store_cols(unsigned char* dst, unsigned char* image, int row, int c, const uint32_t* w)
 {
-    uint4 u[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        __nv_bfloat162 b[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = __floats2bfloat162_rn(v[8 * h + 2 * j], v[8 * h + 2 * j + 1]);
-        u[h] = *reinterpret_cast<uint4*>(b);
-    }
     const uint32_t o = sbuf_off(row, c, C);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        *reinterpret_cast<uint4*>(dst + o + 128 * h) = u[h];
-        if (TRAIN) __stcs(reinterpret_cast<uint4*>(image + o + 128 * h), u[h]);
-    }
-}
-
-__device__ __forceinline__ void add_bias(float* v, const float* b)
-{
-#pragma unroll
-    for (int j = 0; j < 16; j += 4) {
-        const float4 w = *reinterpret_cast<const float4*>(b + j);
-        v[j] += w.x;
-        v[j + 1] += w.y;
-        v[j + 2] += w.z;
-        v[j + 3] += w.w;
+    sts_row16(smem_u32(dst) + o, w);
+    if (TRAIN) {
+        __stcs(reinterpret_cast<uint4*>(image + o), make_uint4(w[0], w[1], w[2], w[3]));
+        __stcs(reinterpret_cast<uint4*>(image + o + 128), make_uint4(w[4], w[5], w[6], w[7]));
     }
 }
 
 // Accumulator columns [c0, c1) of this thread's row + bias, ReLU, stored as
-// BF16 into the canonical buffer (C columns) and its image; bit j of the 16-bit
-// mask half mask[c / 16] is set where column c + j is positive (mask: the row's
-// halves in shared memory; training).
+// BF16 into the canonical buffer (C columns) and its image; training, bits j and
+// 16 + j of the row's mask word of columns [c, c + 16) (kRows words apart, in
+// shared memory) are set where columns c + 2 j and c + 2 j + 1 are positive.
 template <bool TRAIN, int C>
 __device__ __forceinline__ void relu_epilogue(uint32_t tl, const float* bias, unsigned char* dst,
-                                              unsigned char* image, int row, int c0, int c1, uint16_t* mask)
+                                              unsigned char* image, int row, int c0, int c1, uint32_t* mask)
 {
     float v[16];
+    uint32_t w[8];
 #pragma unroll 1
     for (int c = c0; c < c1; c += 16) {
         tmem_ld16(tl + c, v);
-        add_bias(v, bias + c);
-        uint32_t bits = 0;
+        relu16(v, bias + c, w);
+        if (TRAIN) {
+            uint32_t bits = 0;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            v[j] = fmaxf(v[j], 0.f);
-            if (TRAIN) bits |= (v[j] > 0.f ? 1u : 0u) << j;
+            for (int j = 0; j < 8; ++j) bits |= positive2(w[j]) & (0x10001u << j);
+            mask[c / 16 * kRows] = bits;
         }
-        if (TRAIN) mask[c / 16] = (uint16_t)bits;
-        store_cols<TRAIN, C>(dst, image, row, c, v);
+        store_cols<TRAIN, C>(dst, image, row, c, w);
     }
 }
 
 // Accumulator columns [c0, c1) times the ReLU mask, stored as BF16 (the
 // backward through a ReLU layer).
 template <int C>
-__device__ __forceinline__ void mask_epilogue(uint32_t tl, const uint16_t* mask, unsigned char* dst,
+__device__ __forceinline__ void mask_epilogue(uint32_t tl, const uint32_t* mask, unsigned char* dst,
                                               unsigned char* image, int row, int c0, int c1)
 {
     float v[16];
+    uint32_t w[8];
 #pragma unroll 1
     for (int c = c0; c < c1; c += 16) {
         tmem_ld16(tl + c, v);
-        const uint32_t bits = mask[c / 16];
+        const uint32_t bits = mask[c / 16 * kRows];
+        pack16(v, w);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = ((bits >> j) & 1u) ? v[j] : 0.f;
-        store_cols<true, C>(dst, image, row, c, v);
+        for (int j = 0; j < 8; ++j) w[j] &= ((bits >> j) & 0x10001u) * 0xFFFFu;
+        store_cols<true, C>(dst, image, row, c, w);
     }
 }
 
@@ -196,7 +178,7 @@ __device__ __forceinline__ float4 part_lse(uint32_t tz, const float* b3, int c0,
 #pragma unroll 1
     for (int c = c0; c < c1 && c < ncb; c += 16) {
         tmem_ld16(tz + c, v);
-        add_bias(v, b3 + c);
+        add_bias16(v, b3 + c);
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             const float z = v[j];
@@ -225,7 +207,9 @@ __device__ __forceinline__ void store_x(unsigned char* sX, unsigned char* image,
     float v[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) v[c] = c < 8 ? x[c] : (c == 8 ? 1.f : 0.f);
-    store_cols<TRAIN, 16>(sX, image, row, 0, v);
+    uint32_t w[8];
+    pack16(v, w);
+    store_cols<TRAIN, 16>(sX, image, row, 0, w);
 }
 
 template <bool TRAIN>
@@ -244,8 +228,8 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
     uint32_t* const slot = reinterpret_cast<uint32_t*>(sm + kSSlot);
     const int tid = threadIdx.x, row = tid & (kRows - 1), part = tid / kRows;
     const bool issuer = warp_uniform(threadIdx.x >> 5) == 0;    // the warp of the MMAs and the bulk stores
-    uint16_t* const m1 = reinterpret_cast<uint16_t*>(sm + kSMask) + row * 24;   // h1: 8 halves
-    uint16_t* const m2 = m1 + 8;                                                // h2: 16 halves
+    uint32_t* const m1 = reinterpret_cast<uint32_t*>(sm + kSMask) + row;        // h1: 8 words, kRows apart
+    uint32_t* const m2 = m1 + 8 * kRows;                                        // h2: 16 words
     const int ncb = a.ncb;
     const bool halves = ncb > 128;
     const uint32_t w3bytes = halves ? kW3Half : (uint32_t)ncb * kW2 * 2;
@@ -395,12 +379,14 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
                 for (int c = zc0; c < zc1; c += 16) {
                     if (c < ncb) {
                         tmem_ld16(tl + kTZ + c, v);
-                        add_bias(v, b3s + c);
+                        add_bias16(v, b3s + c);
                     }
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
                         v[j] = c < ncb ? g * (__expf(v[j] - lse) - (c + j == t ? 1.f : 0.f)) : 0.f;
-                    store_cols<TRAIN, 128>(sA, blob + kBZ, row, c, v);
+                    uint32_t w[8];
+                    pack16(v, w);
+                    store_cols<TRAIN, 128>(sA, blob + kBZ, row, c, w);
                 }
             }
         }

@@ -9,8 +9,8 @@
 // another.  Four warpgroups serve the tile's 128 rows (TMEM lanes), each
 // taking 32 of every 128-column epilogue's columns; the loss epilogue is
 // warpgroup 0's.  Warp 0 issues each tcgen05.mma round; after it completes,
-// all threads run its epilogue (bias, ReLU and its mask, BF16 into shared
-// memory):
+// all threads run its epilogue (bias and ReLU, or the ReLU's mask, BF16 into
+// shared memory):
 //   forward  H1 = relu(X W1^T + b1), H2, H3, Z = H3 W4^T + b4 (FP32 accumulation)
 //   loss     per row: diff = Z - s_G, n = |diff|; dZ = lambda/n_total diff/n;
 //            d_feat -= lambda/n_total max(u, w_s) diff/n (added to the caller's array)
@@ -63,8 +63,7 @@ constexpr uint32_t kOH3 = kOH2 + sbuf_bytes(128, 128);
 constexpr uint32_t kODZ = kOH3 + sbuf_bytes(128, 128);       // [128][16]
 constexpr uint32_t kOE = kODZ + sbuf_bytes(128, 16);         // [128][16], column 0 = 1
 constexpr uint32_t kOB = kOE + sbuf_bytes(128, 16);          // biases FP32: b1, b2, b3 (128 each), b4 (8)
-constexpr uint32_t kOM = kOB + (3 * kH + 16) * 4;           // ReLU masks: [3 layers][4 words][128 rows] u32
-constexpr uint32_t kOBar = kOM + 3 * 4 * 128 * 4;
+constexpr uint32_t kOBar = kOB + (3 * kH + 16) * 4;
 constexpr uint32_t kSmoothSmem = kOBar + 32 + 1024;
 
 struct Ctx {
@@ -99,46 +98,32 @@ __device__ __forceinline__ void publish()
 }
 
 // This warpgroup's 32 columns of the epilogue of a 128-column hidden layer:
-// v = acc + b; relu; BF16 into H; the ReLU mask bits into mask[part * 128 + row].
-__device__ __forceinline__ void hidden_epilogue(const Ctx& c, const float* b, uint32_t hoff, uint32_t* mask)
+// relu(acc + b) in BF16 into H.
+__device__ __forceinline__ void hidden_epilogue(const Ctx& c, const float* b, uint32_t hoff)
 {
-    const SBuf Hs{c.sm + hoff, kH};
-    {
-        const int q = 2 * c.part;
-        uint32_t mw = 0;
+    float v[16];
+    uint32_t w[8];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[16];
-            tmem_ld16(c.tmem + c.lanef + kAcc + 16 * (q + h), v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float x = v[j] + b[16 * (q + h) + j];
-                mw |= (x > 0.f ? 1u : 0u) << (16 * h + j);
-                v[j] = fmaxf(x, 0.f);
-            }
-            sbuf_store8(Hs, c.row, 16 * (q + h), v);
-            sbuf_store8(Hs, c.row, 16 * (q + h) + 8, v + 8);
-        }
-        mask[(q >> 1) * 128 + c.row] = mw;
+    for (int q = 0; q < 2; ++q) {
+        const int col = 32 * c.part + 16 * q;
+        tmem_ld16(c.tmem + c.lanef + kAcc + col, v);
+        relu16(v, b + col, w);
+        sts_row16(c.s0 + hoff + sbuf_off(c.row, col, kH), w);
     }
 }
 
-// This warpgroup's 32 columns of a backward epilogue: dH = acc o mask, BF16 into H's buffer.
-__device__ __forceinline__ void grad_epilogue(const Ctx& c, uint32_t hoff, const uint32_t* mask)
+// This warpgroup's 32 columns of a backward epilogue: dH = acc o [H > 0], BF16 over H.
+__device__ __forceinline__ void grad_epilogue(const Ctx& c, uint32_t hoff)
 {
-    const SBuf Hs{c.sm + hoff, kH};
-    {
-        const int q = 2 * c.part;
-        const uint32_t mw = mask[(q >> 1) * 128 + c.row];
+    float v[16];
+    uint32_t w[8];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[16];
-            tmem_ld16(c.tmem + c.lanef + kAcc + 16 * (q + h), v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = ((mw >> (16 * h + j)) & 1u) ? v[j] : 0.f;
-            sbuf_store8(Hs, c.row, 16 * (q + h), v);
-            sbuf_store8(Hs, c.row, 16 * (q + h) + 8, v + 8);
-        }
+    for (int q = 0; q < 2; ++q) {
+        const int col = 32 * c.part + 16 * q;
+        const uint32_t at = c.s0 + hoff + sbuf_off(c.row, col, kH);
+        tmem_ld16(c.tmem + c.lanef + kAcc + col, v);
+        relu_mask16(v, at, w);
+        sts_row16(at, w);
     }
 }
 
@@ -300,21 +285,18 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
             sbuf_store8(SBuf{c.sm + kOX, 16}, c.row, 0, v);
             sbuf_store8(SBuf{c.sm + kOX, 16}, c.row, 8, z);
         }
-        uint32_t* m1 = reinterpret_cast<uint32_t*>(c.sm + kOM);
-        uint32_t* m2 = m1 + 4 * 128;
-        uint32_t* m3 = m2 + 4 * 128;
         publish();
         issue(c, 0, first);
         if (!(ok = round_wait(c))) break;
-        hidden_epilogue(c, b1, kOH1, m1);
+        hidden_epilogue(c, b1, kOH1);
         publish();
         issue(c, 1, first);
         if (!(ok = round_wait(c))) break;
-        hidden_epilogue(c, b2, kOH2, m2);
+        hidden_epilogue(c, b2, kOH2);
         publish();
         issue(c, 2, first);
         if (!(ok = round_wait(c))) break;
-        hidden_epilogue(c, b3, kOH3, m3);
+        hidden_epilogue(c, b3, kOH3);
         publish();
         issue(c, 3, first);
         if (!(ok = round_wait(c))) break;
@@ -346,15 +328,15 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
         publish();
         issue(c, 4, first);
         if (!(ok = round_wait(c))) break;
-        grad_epilogue(c, kOH3, m3);              // dH3 over H3 (read by dW4, complete)
+        grad_epilogue(c, kOH3);              // dH3 over H3 (read by dW4, complete)
         publish();
         issue(c, 5, first);
         if (!(ok = round_wait(c))) break;
-        grad_epilogue(c, kOH2, m2);              // dH2 over H2
+        grad_epilogue(c, kOH2);              // dH2 over H2
         publish();
         issue(c, 6, first);
         if (!(ok = round_wait(c))) break;
-        grad_epilogue(c, kOH1, m1);              // dH1 over H1
+        grad_epilogue(c, kOH1);              // dH1 over H1
         publish();
         issue(c, 7, first);
         if (!(ok = round_wait(c))) break;
