@@ -52,10 +52,8 @@ struct DecArgs {
     float *dW1, *db1, *dW2, *db2, *dW3, *db3;
     int32_t* argmax;
     float* prob;
-    // feature-map export: W3 as the BF16 shared-memory image (reloaded per tile
-    // when the output staging borrows W3's shared memory)
+    // query: W3 as its BF16 shared-memory image
     const unsigned char* W3_img;
-    int w3_reload;
     // query
     const unsigned char* G_img;     // ncb/64 chunks of [ncb x 64] canonical bf16
     const float* Aq;                // [16, ncb] fp32 = [text; negs] S_c^T
@@ -63,7 +61,6 @@ struct DecArgs {
     float* rel;
     // feature-map export
     int dd;                         // feature dims d (multiple of 64)
-    __nv_bfloat16* fmap;            // [P, dd] out
     // training with the RGB L1 term of the same pixels (nullable img): img, img_t [3, P],
     // d_img [3, P] = sign(img - img_t) inv_l1, *loss_l1 += sum |img - img_t| inv_l1
     const float *img, *img_t;
@@ -1040,209 +1037,289 @@ __global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecAr
 // ---------------------------------------------------------------------------
 // Language feature map export F = M_infer S (supp. Sec. "Inference"): per
 // pixel the decoder's softmax p over the n_cb codes times the codebook, in
-// BF16.  Four warpgroups serve the same 128 rows as in the query kernel; e =
-// exp(z - max z) is stored in BF16 and each output row is scaled by 1/sum e.
-// The codebook streams through shared memory in 64-dim chunks ([n_cb x 64]
-// canonical images, two slots, 1-D bulk copies); per chunk one MMA (M = 128
-// pixels, N = 64 dims, K = n_cb) reads the chunk MN-major into one of two
-// 64-column TMEM accumulators.  Each warpgroup converts 16 columns of each
-// into a 128-byte-swizzled staging area, from which two TMA tensor stores per
-// round (128 pixels x 64 dims each) write the output in whole lines; a warp
-// storing its rows directly would scatter 16-byte pieces over 32 rows.
-constexpr uint32_t kTF = 256;      // TMEM columns of the two chunk accumulators
+// BF16; e = exp(z - max z) is rounded to BF16 and each output row is scaled by
+// 1 / sum e.  Two 128-pixel tiles are in flight per CTA, each with its own two
+// warpgroups, MMA warp and load warp, going through two phases:
+//   front  the warpgroups decode the tile and write e over its logits in tensor
+//          memory, as the A operand of
+//   back   F = e S in 128-dim chunks.  The codebook streams through the tile's
+//          four 8 KB slots ([32 codes x 128 dims], bulk copies), the MMA warp
+//          contracts them into 128 TMEM columns, and the warpgroups drain a
+//          finished chunk, 64 dims each, through two 64-byte-swizzled staging
+//          boxes and TMA tensor stores (128 pixels x 32 dims).
+// The second tile starts when the first one enters its back phase, so one tile's
+// front, bound by the latency of its rounds, runs beside the other's MMAs and
+// stores.  e in tensor memory leaves shared memory for the slots; N = 128 because
+// an MMA of N = 64 takes three quarters as long.  A 1296 x 840 view at 256 codes:
+// 0.679 ms (2.9 TB/s written); two tiles in phase sharing every slot 0.812 ms, the
+// same with e in shared memory 0.886 ms, one tile at a time in rounds of two
+// 64-dim chunks 1.255 ms.  Per tile, 45,000 cycles: 17,000 in the front, 13,000
+// waiting for the codebook (the latency of four slots), 13,000 of MMAs.
+constexpr int kXSlots = 4, kXCodes = 32, kXDims = 128;
+constexpr uint32_t kXSlotBytes = sbuf_bytes(kXCodes, kXDims), kXBox = sbuf_bytes(128, 32);
+// A tile's region: X1 and H1, then H2 over them; in the back phase two staging boxes per warpgroup.
+constexpr uint32_t kXAct = sbuf_bytes(128, 128);
+static_assert(kXAct == 4 * kXBox && kXAct >= sbuf_bytes(128, 16) + sbuf_bytes(128, 64), "export region");
+constexpr int kXThreads = 4 * 128 + 4 * 32;
+constexpr uint32_t kXAcc = 128;              // TMEM columns of a tile's 256: e in [0, ncb / 2), the accumulator
 
-// Shared memory of the export kernel without the output staging, the staging
-// (one round's two 128 x 64 BF16 boxes, 128-byte swizzled for the TMA store),
-// and whether the staging must borrow W3's shared memory (then W3 is reloaded
-// from its global image after every tile; it is idle during the codebook loop).
-// The layout starts at a 1024-byte boundary (the swizzled staging and W3s, at
-// offset 18 KB, need it), hence the first 1024.
-__host__ constexpr size_t export_smem_core(int ncb)
-{
-    return 1024 + weights_bytes(ncb) + (sbuf_bytes(128, ncb) > kFwdWgBytes ? sbuf_bytes(128, ncb) : kFwdWgBytes) +
-           2 * sbuf_bytes(ncb, 64) + kQueryParts * 128 * 4 + 128;
-}
-constexpr uint32_t kExportBox = sbuf_bytes(128, 64);
-constexpr size_t kMaxDynSmem = 227 * 1024;
-__host__ constexpr bool export_stage_in_w3(int ncb) { return export_smem_core(ncb) + 1024 + 2 * kExportBox > kMaxDynSmem; }
+struct ExportBars {                          // of one tile slot
+    uint64_t full[kXSlots], empty[kXSlots];  // codebook slots
+    uint64_t acc_full, acc_free;             // a chunk's accumulator
+    uint64_t e_ready;                        // the tile's e is in tensor memory
+    uint64_t front, fin;
+};
+
+// The layout starts at a 1024-byte boundary.
 __host__ constexpr size_t export_smem(int ncb)
 {
-    return export_smem_core(ncb) + (export_stage_in_w3(ncb) ? 0 : 1024 + 2 * kExportBox);
+    return 1024 + 2 * kXAct + 2 * kXSlots * kXSlotBytes + weights_bytes(ncb) + 4 * 128 * 4 + 256;
 }
+static_assert(export_smem(256) <= 227 * 1024 && 2 * sizeof(ExportBars) + 4 <= 256, "export shared memory");
 
-__global__ void __launch_bounds__(128 * kQueryParts, 1) export_fused_kernel(const __grid_constant__ CUtensorMap tmap_out,
-                                                                          DecArgs a)
+__global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid_constant__ CUtensorMap tmap_out,
+                                                                    DecArgs a)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char* const act =
+        reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm) + 1023) & ~uintptr_t(1023));
+    unsigned char* const slots0 = act + 2 * kXAct;
+    const int ncb = a.ncb;
     Front f;
-    unsigned char* p = load_weights(
-        reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm) + 1023) & ~uintptr_t(1023)), a, f);
-    f.X1 = SBuf{p, 16};
-    f.H1 = SBuf{p + sbuf_bytes(128, 16), 64};
-    f.H2 = SBuf{p + sbuf_bytes(128, 16) + sbuf_bytes(128, 64), 128};
-    const SBuf Ps{p, a.ncb};
-    f.xch = reinterpret_cast<float4*>(p);
-    p += sbuf_bytes(128, a.ncb) > kFwdWgBytes ? sbuf_bytes(128, a.ncb) : kFwdWgBytes;
-    const uint32_t chunk_bytes = sbuf_bytes(a.ncb, 64);
-    const SBuf Gs[2] = {SBuf{p, 64}, SBuf{p + chunk_bytes, 64}};
-    p += 2 * chunk_bytes;
-    float* sums = reinterpret_cast<float*>(p);          // [parts][128] partial sums of e
-    p += kQueryParts * 128 * 4;
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(p);     // [0] MMA, [1], [2] codebook slots, [4] W3 reload
-    uint32_t* slot = reinterpret_cast<uint32_t*>(p + 24);
-    p += 128;
-    unsigned char* stg = a.w3_reload ? f.W3s.p
-                                     : reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(p) + 1023) &
-                                                                        ~uintptr_t(1023));
-    const int tid = threadIdx.x;
-    f.mbar = mbar;
-    f.phase = 0;
-    f.tid = tid & 127;
-    f.bar_id = 0;
-    f.nthreads = blockDim.x;
-    const int warp = (int)warp_uniform(threadIdx.x >> 5);
-    f.half = warp >> 2;
-    f.issuer = warp == 0;
-    f.nhalf = kQueryParts;
-    f.w3bar = mbar + 4;
-    if (tid == 0) {
-        for (int i = 0; i < 3; ++i) mbar_init(mbar + i, 1);
-        mbar_init(mbar + 4, 1);
+    unsigned char* p = load_weights(slots0 + 2 * kXSlots * kXSlotBytes, a, f);
+    float* const sums = reinterpret_cast<float*>(p);              // [tile slot][half][128] partial sums of e
+    p += 4 * 128 * 4;
+    ExportBars* const bars = reinterpret_cast<ExportBars*>(p);    // [tile slot]
+    uint32_t* const tslot = reinterpret_cast<uint32_t*>(bars + 2);
+    if (threadIdx.x < 2) {
+        ExportBars* const b = bars + threadIdx.x;
+        for (int i = 0; i < kXSlots; ++i) {
+            mbar_init(b->full + i, 1);
+            mbar_init(b->empty + i, 1);
+        }
+        mbar_init(&b->acc_full, 1);
+        mbar_init(&b->acc_free, 8);
+        mbar_init(&b->e_ready, 1);
+        mbar_init(&b->front, 1);
+        mbar_init(&b->fin, 1);
     }
-    if (tid < 32) tmem_alloc(slot, 512);
+    const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (warp == 0) tmem_alloc(tslot, 512);
     fence_proxy_async();
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
-    f.tw = tbase;
-    f.lane = (uint32_t)(32 * ((tid >> 5) & 3)) << 16;
-    const int row = f.tid;
-    int c0, c1;
-    my_cols(f, a.ncb, c0, c1);
-    const int nch = a.dd / 64;
-    uint32_t gphase[2] = {0u, 0u};
-    bool pending[2] = {false, false};
-    auto load_chunk = [&](int kc, int s) {
-        mbar_expect_tx(mbar + 1 + s, chunk_bytes);
-        bulk_g2s(Gs[s].p, a.G_img + (size_t)kc * chunk_bytes, chunk_bytes, mbar + 1 + s);
-        pending[s] = true;
-    };
+    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(tslot));
     const int ntiles = (a.P + 127) / 128;
+    const int nch = (a.dd + kXDims - 1) / kXDims, nkb = (ncb + kXCodes - 1) / kXCodes;
+    const auto width = [&](int j) { return min(kXDims, a.dd - j * kXDims); };        // 128, or 64 in the last chunk
+    const auto codes = [&](int k) { return min(kXCodes, ncb - k * kXCodes); };       // 32, or 16 in the last block
+    // tile slot t takes the tiles blockIdx.x + gridDim.x (t + 2 i)
+    const int t = warp < 16 ? warp >> 3 : warp & 1;
+    const int first = blockIdx.x + gridDim.x * t, stride = 2 * gridDim.x;
+    ExportBars* const bar = bars + t;
+    unsigned char* const slots = slots0 + t * kXSlots * kXSlotBytes;
+    const uint32_t td = tbase + 256u * t;
     bool ok = true;
-    if (tid == 0 && blockIdx.x < ntiles)
-        for (int s = 0; s < 2 && s < nch; ++s) load_chunk(s, s);
-    float xf[8];                                // this tile's R_s, loaded a tile ahead (part 0)
-    if (f.half == 0) load_feat(a, blockIdx.x * 128 + row, blockIdx.x * 128 + row < a.P, xf);
-    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int px = tile * 128 + row;
-        const bool valid = px < a.P;
-        if (!mlp_forward_x(f, a, xf)) break;
-        if (f.half == 0) {
-            const int nx = px + 128 * (int)gridDim.x;
-            load_feat(a, nx, tile + (int)gridDim.x < ntiles && nx < a.P, xf);
-        }
-        float v[16], mh = -INFINITY;
-        for (int c = c0; c < c1; c += 16) {
-            tmem_ld16(f.tw + f.lane + c, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) mh = fmaxf(mh, v[j] + f.b3s[c + j]);
-        }
-        f.xch[f.half * 128 + row].x = mh;
-        wg_sync(f);
-        float m = -INFINITY;
-#pragma unroll
-        for (int h = 0; h < kQueryParts; ++h) m = fmaxf(m, f.xch[h * 128 + row].x);
-        wg_sync(f);
-        const float ml = m * 1.4426950408889634f;
-        float se = 0.f;
-        for (int c = c0; c < c1; c += 16) {
-            tmem_ld16(f.tw + f.lane + c, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                v[j] = ex2_approx(fmaf(v[j] + f.b3s[c + j], 1.4426950408889634f, -ml));
-                se += v[j];
-            }
-            sbuf_store8(Ps, row, c, v);
-            sbuf_store8(Ps, row, c + 8, v + 8);
-        }
-        sums[f.half * 128 + row] = se;
-        wg_publish(f);
-        float tot = 0.f;
-#pragma unroll
-        for (int h = 0; h < kQueryParts; ++h) tot += sums[h * 128 + row];
-        const float inv = valid ? 1.0f / tot : 0.f;
-        bool tmo = false;
-        for (int kc0 = 0; kc0 < nch; kc0 += 2) {
-            if (tid == 0) {
-                for (int s = 0; s < 2 && kc0 + s < nch; ++s) {
-                    if (!mbar_wait(mbar + 1 + s, gphase[s])) tmo = true;
-                    gphase[s] ^= 1u;
-                    pending[s] = false;
-                    const uint64_t gm = mndesc(Gs[s], 0, 0);
-                    for (int k = 0; k < a.ncb / 16; ++k)
-                        mma(tbase + kTF + 64 * s, kdesc(Ps, 0, 16 * k), gm + 128 * k, idesc_bf16(64, false, true),
-                            k > 0);
-                }
-                commit(f.mbar);
-                // the staging area is rewritten below: the previous round's stores must have read it
-                bulk_wait_read_all();
-            }
-            if (!wg_wait(f) || bar_any(0, blockDim.x, tmo)) {
-                if (tid == 0) atomicExch(&g_tc_error, 1);
-                ok = false;
-                break;
-            }
-            // refill the slots: the next chunk pair of this tile, or the first pair of the next tile
-            if (tid == 0) {
-                const bool more = kc0 + 2 < nch;
-                const bool next_tile = tile + (int)gridDim.x < ntiles;
-                for (int s = 0; s < 2; ++s) {
-                    const int kc = more ? kc0 + 2 + s : s;
-                    if ((more && kc < nch) || (!more && next_tile && kc < nch)) load_chunk(kc, s);
+
+    if (warp >= 18) {
+        // the codebook, chunk by chunk, for every tile of the slot
+        uint32_t it = 0;
+        for (int tile = first; tile < ntiles && ok; tile += stride)
+            for (int j = 0; j < nch && ok; ++j) {
+                const uint32_t row = (uint32_t)width(j) * 2;
+                const unsigned char* src = a.G_img + (size_t)j * ncb * kXDims * 2;
+                for (int k = 0; k < nkb; ++k, ++it) {
+                    const uint32_t sl = it % kXSlots;
+                    if (it >= kXSlots &&
+                        !(ok = warp_agree(mbar_wait(bar->empty + sl, (it / kXSlots - 1) & 1u))))
+                        break;
+                    if (elect_one()) {
+                        mbar_expect_tx(bar->full + sl, codes(k) * row);
+                        bulk_g2s(slots + sl * kXSlotBytes, src + (size_t)k * kXCodes * row, codes(k) * row,
+                                 bar->full + sl);
+                    }
+                    __syncwarp();
                 }
             }
-            // this warpgroup's 16 columns of each chunk, scaled by 1 / sum e, as BF16 into the
-            // staging boxes (row-major 128-byte rows, 16-byte unit u of row r at u ^ (r & 7))
-            for (int s = 0; s < 2 && kc0 + s < nch; ++s) {
-                tmem_ld16(tbase + kTF + 64 * s + 16 * f.half + f.lane, v);
-                __nv_bfloat162 h[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(v[2 * j] * inv, v[2 * j + 1] * inv);
-                unsigned char* dst = stg + s * kExportBox + row * 128;
-                const int u = 2 * f.half;
-                *reinterpret_cast<uint4*>(dst + ((u ^ (row & 7)) << 4)) = *reinterpret_cast<uint4*>(h);
-                *reinterpret_cast<uint4*>(dst + (((u + 1) ^ (row & 7)) << 4)) = *reinterpret_cast<uint4*>(h + 4);
+        // copies still in flight land before the shared memory goes away
+        for (uint32_t i = it - min(it, (uint32_t)kXSlots); i < it; ++i)
+            ok = mbar_wait(bar->full + i % kXSlots, (i / kXSlots) & 1u) && ok;
+    } else if (warp >= 16) {
+        // the back phase's MMAs
+        uint32_t it = 0, r = 0, c = 0;
+        const uint32_t slots_a = smem_u32(slots);
+        for (int tile = first; tile < ntiles && ok; tile += stride, ++r) {
+            if (!(ok = warp_agree(mbar_wait(&bar->e_ready, r & 1u)))) break;
+            for (int j = 0; j < nch && ok; ++j, ++c) {
+                const uint32_t C = (uint32_t)width(j), id = idesc_bf16((int)C, false, true);
+                if (c >= 1 && !(ok = warp_agree(mbar_wait(&bar->acc_free, (c - 1) & 1u)))) break;
+                fence_after();
+                for (int k = 0; k < nkb; ++k, ++it) {
+                    const uint32_t sl = it % kXSlots;
+                    if (!(ok = warp_agree(mbar_wait(bar->full + sl, (it / kXSlots) & 1u)))) break;
+                    fence_after();
+                    const uint64_t gm = mndesc_at(slots_a + sl * kXSlotBytes, (int)C, 0, 0);
+                    const uint32_t ea = td + 8u * (kXCodes / 16) * k;
+                    const bool two = codes(k) > 16;
+                    if (elect_one()) {
+                        mma_ta(td + kXAcc, ea, gm, id, k > 0);
+                        if (two) mma_ta(td + kXAcc, ea + 8u, gm + 2ull * C, id, 1u);
+                        commit(bar->empty + sl);
+                        if (k + 1 == nkb) commit(&bar->acc_full);
+                    }
+                    __syncwarp();
+                }
             }
-            fence_proxy_async();
+        }
+        if (elect_one()) commit(&bar->fin);
+        ok = mbar_wait(&bar->fin, 0) && ok;
+    } else {
+        // half h of the tile's columns
+        const int wg = warp >> 2;
+        f.half = wg & 1;
+        f.nhalf = 2;
+        f.issuer = (warp & 7) == 0;
+        f.tid = threadIdx.x & 127;
+        f.bar_id = 1 + t;
+        f.nthreads = 256;
+        f.mbar = &bar->front;
+        f.phase = 0;
+        f.tw = td;
+        f.lane = (uint32_t)(32 * (warp & 3)) << 16;
+        unsigned char* const reg = act + t * kXAct;
+        f.X1 = SBuf{reg, 16};
+        f.H1 = SBuf{reg + sbuf_bytes(128, 16), 64};
+        f.H2 = SBuf{reg, 128};
+        f.xch = reinterpret_cast<float4*>(reg);
+        const uint32_t tl = f.tw + f.lane;
+        unsigned char* const stg = act + wg * 2 * kXBox;
+        const int row = f.tid;
+        const bool lead = row == 0;                 // of the warpgroup
+        // e takes half the logits' columns (two codes a word), so writing it in place must not pass unread
+        // logits: each half keeps up to four 16-code units in registers (half 0 its upper ones, whose columns
+        // half 1's e will take; half 1 its first ones) until the other has read that far, then goes on in place
+        const int nu = ncb / 16, nu0 = (nu + 1) / 2;
+        const int u0 = f.half ? nu0 : 0, u1 = f.half ? nu : nu0;
+        const int held = f.half ? min(4, nu - nu0) : nu0 - nu0 / 2, hu = f.half ? nu0 : nu0 / 2;
+        const int rest0 = f.half ? hu + held : 0, rest1 = f.half ? nu : hu;
+        float xf[8];                                // this tile's R_s (half 0), in L2 a tile ahead
+        if (f.half == 0) load_feat(a, first * 128 + row, first < ntiles && first * 128 + row < a.P, xf);
+        // out of phase with the first slot
+        if (t == 1 && first < ntiles) ok = !bar_any(f.bar_id, 256, !mbar_wait(&bars->e_ready, 0));
+        uint32_t c = 0;
+        for (int tile = first; tile < ntiles && ok; tile += stride) {
+            const bool valid = tile * 128 + row < a.P;
+            if (!(ok = mlp_forward_x(f, a, xf))) break;
+            const int nx = tile + stride < ntiles ? (tile + stride) * 128 + row : a.P;
+            const bool more = f.half == 0 && nx < a.P;
+            if (more)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) prefetch_l2(a.feat + (size_t)i * a.P + nx);
+            float v[16], mh = -INFINITY;
+            for (int u = u0; u < u1; ++u) {
+                tmem_ld16(tl + 16 * u, v);
+                add_bias16(v, f.b3s + 16 * u);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) mh = fmaxf(mh, v[j]);
+            }
+            f.xch[f.half * 128 + row].x = mh;
+            wg_sync(f);
+            const float m = fmaxf(f.xch[row].x, f.xch[128 + row].x);
+            const float ml = m * 1.4426950408889634f;
+            float se = 0.f;
+            const auto unit = [&](int u, uint32_t* w) {
+                tmem_ld16(tl + 16 * u, v);
+                add_bias16(v, f.b3s + 16 * u);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    v[j] = ex2_approx(fmaf(v[j], 1.4426950408889634f, -ml));
+                    se += v[j];
+                }
+                pack16(v, w);
+            };
+            uint32_t hold[4][8], w[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < held) unit(hu + i, hold[i]);
             fence_before();
-            __syncthreads();
+            wg_sync(f);
             fence_after();
-            if (tid == 0) {
-                for (int s = 0; s < 2 && kc0 + s < nch; ++s)
-                    tma_store_2d(&tmap_out, 64 * (kc0 + s), tile * 128, stg + s * kExportBox);
-                bulk_commit();
-                // after the tile's last round, W3 goes back into the staging area for the next tile
-                if (a.w3_reload && kc0 + 2 >= nch && tile + (int)gridDim.x < ntiles) {
-                    bulk_wait_read_all();
-                    mbar_expect_tx(f.w3bar, sbuf_bytes(a.ncb, 128));
-                    bulk_g2s(f.W3s.p, a.W3_img, sbuf_bytes(a.ncb, 128), f.w3bar);
-                    f.w3pending = true;
+            if (f.half) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < held) tmem_st8(tl + 8 * (hu + i), hold[i]);
+            }
+            for (int u = rest0; u < rest1; ++u) {
+                unit(u, w);
+                tmem_st8(tl + 8 * u, w);
+            }
+            if (!f.half) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < held) tmem_st8(tl + 8 * (hu + i), hold[i]);
+            }
+            tmem_wait_st();
+            sums[wg * 128 + row] = se;
+            fence_before();
+            wg_sync(f);
+            fence_after();
+            if (lead && f.half == 0) mbar_arrive(&bar->e_ready);
+            const float inv = valid ? 1.0f / (sums[2 * t * 128 + row] + sums[(2 * t + 1) * 128 + row]) : 0.f;
+            for (int j = 0; j < nch; ++j, ++c) {
+                const bool got = mbar_wait(&bar->acc_full, c & 1u);
+                // every thread of the tile leaves together
+                if (bar_any(f.bar_id, 256, !got)) {
+                    ok = false;
+                    break;
+                }
+                fence_after();
+                const bool mine = 64 * f.half < width(j);
+                __nv_bfloat162 h[32];
+                if (mine) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        tmem_ld16(tl + kXAcc + 64u * f.half + 16u * q, v);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            h[8 * q + i] = __floats2bfloat162_rn(v[2 * i] * inv, v[2 * i + 1] * inv);
+                    }
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bar->acc_free);
+                if (!mine) continue;
+                // row-major 64-byte rows, 16-byte unit u of row r at u ^ ((r >> 1) & 3); a box is rewritten once
+                // the store before the last one has read it
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    if (lead) bulk_wait_read_but_one();
+                    asm volatile("bar.sync %0, 128;" ::"r"(3 + wg) : "memory");
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        *reinterpret_cast<uint4*>(stg + q * kXBox + row * 64 + ((u ^ ((row >> 1) & 3)) << 4)) =
+                            *reinterpret_cast<uint4*>(h + 16 * q + 4 * u);
+                    fence_proxy_async();
+                    asm volatile("bar.sync %0, 128;" ::"r"(3 + wg) : "memory");
+                    if (lead) {
+                        tma_store_2d(&tmap_out, kXDims * j + 64 * f.half + 32 * q, tile * 128, stg + q * kXBox);
+                        bulk_commit();
+                    }
                 }
             }
+            if (!ok) break;
+            if (f.half == 0) load_feat(a, nx, more, xf);
+            // the next tile's X1 and H1 go where the staging boxes are
+            if (lead) bulk_wait_read_all();
+            wg_sync(f);
         }
-    }
-    // drain copies still in flight before the shared memory goes away
-    if (tid == 0) {
-        for (int s = 0; s < 2; ++s)
-            if (pending[s]) mbar_wait(mbar + 1 + s, gphase[s]);
-        if (f.w3pending) mbar_wait(f.w3bar, f.w3phase);
-        bulk_wait_all();
+        if (lead) bulk_wait_all();
     }
     fence_before();
-    __syncthreads();
+    const bool bad = __syncthreads_or(!ok);
     fence_after();
-    if (tid < 32) tmem_dealloc(tbase, 512);
+    if (bad && threadIdx.x == 0) atomicExch(&g_tc_error, 1);
+    if (warp == 0) tmem_dealloc(tbase, 512);
 }
 
 // W3 [ncb x 128] (fp32) -> its BF16 shared-memory image (the layout load_weights writes).
@@ -1257,20 +1334,20 @@ __global__ void w3_image_kernel(const float* __restrict__ W3, int ncb, unsigned 
     }
 }
 
-// Codebook S [ncb x dd] (fp32) -> chunked canonical bf16 image: chunk kc holds
-// dims [64 kc, 64 kc + 64) of every code, as an [ncb x 64] canonical buffer.
+// The export's codebook S [ncb x dd] (fp32) as a chunked canonical BF16 image:
+// chunk j holds dims [128 j, 128 j + 128) (64 in the last chunk of an odd multiple
+// of 64) of every code, as an [ncb x 128] canonical buffer, whose blocks of 64
+// codes are contiguous.
 __global__ void codebook_chunks_kernel(const float* __restrict__ S, int ncb, int dd, unsigned char* __restrict__ img)
 {
     const int n8 = ncb * (dd / 8);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += gridDim.x * blockDim.x) {
-        const int r = i / (dd / 8), c0 = (i % (dd / 8)) * 8;
-        const int kc = c0 / 64, cc = c0 % 64;
-        __nv_bfloat162 h[4];
+        const int r = i / (dd / 8), c0 = (i % (dd / 8)) * 8, j = c0 / kXDims;
+        float v[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            h[j] = __floats2bfloat162_rn(S[(size_t)r * dd + c0 + 2 * j], S[(size_t)r * dd + c0 + 2 * j + 1]);
-        unsigned char* dst = img + (size_t)kc * ncb * 64 * 2 + ((r >> 3) * 8 * 128 + (cc >> 3) * 128 + (r & 7) * 16);
-        *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<uint4*>(h);
+        for (int k = 0; k < 8; ++k) v[k] = S[(size_t)r * dd + c0 + k];
+        const SBuf dst{img + (size_t)j * ncb * kXDims * 2, min(kXDims, dd - j * kXDims)};
+        sbuf_store8(dst, r, c0 - j * kXDims, v);
     }
 }
 
@@ -1483,17 +1560,16 @@ le_status export_fused(int32_t P, const float* feat, const le_decoder* d, const 
     if (st != LE_OK) return st;
     const int ncb = d->n_cb;
     unsigned char* img = static_cast<unsigned char*>(ws);
-    unsigned char* w3img = img + (size_t)ncb * dd * 2;
-    // output tensor map: [P rows, dd columns] BF16, boxes of 128 rows x 64 columns, 128-byte swizzle
+    // output tensor map: [P rows, dd columns] BF16, boxes of 128 rows x 32 columns, 64-byte swizzle
     EncodeTiled enc;
     if ((st = tensor_map_encoder(&enc)) != LE_OK) return st;
     CUtensorMap tmap;
     const cuuint64_t dims[2] = {(cuuint64_t)dd, (cuuint64_t)P};
     const cuuint64_t strides[1] = {(cuuint64_t)dd * 2};
-    const cuuint32_t box[2] = {64, 128};
+    const cuuint32_t box[2] = {32, 128};
     const cuuint32_t estr[2] = {1, 1};
     if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, out, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
+            CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
         CUDA_SUCCESS) {
         set_error("cuTensorMapEncodeTiled failed for the feature map");
         return LE_ERR_CUDA;
@@ -1507,22 +1583,10 @@ le_status export_fused(int32_t P, const float* feat, const le_decoder* d, const 
     a.W1 = d->W1; a.b1 = d->b1; a.W2 = d->W2; a.b2 = d->b2; a.W3 = d->W3; a.b3 = d->b3;
     a.G_img = img;
     a.dd = dd;
-    a.fmap = out;
-    a.w3_reload = export_stage_in_w3(ncb) ? 1 : 0;
-    if (a.w3_reload && sbuf_bytes(ncb, 128) < 2 * kExportBox) {
-        set_error("feature map export: no shared memory for the output staging with n_cb = %d", ncb);
-        return LE_ERR_UNSUPPORTED;
-    }
-    if (a.w3_reload) {
-        w3_image_kernel<<<16, 256, 0, s>>>(d->W3, ncb, w3img);
-        LE_LAUNCHED();
-        a.W3_img = w3img;
-    }
     const size_t smem = export_smem(ncb);
     if ((st = set_smem(export_fused_kernel, smem)) != LE_OK) return st;
-    const int ntiles = (P + 127) / 128;
-    const int grid = ntiles < sm_count() ? ntiles : sm_count();
-    export_fused_kernel<<<grid, 128 * kQueryParts, smem, s>>>(tmap, a);
+    const int ntiles = (P + 127) / 128, sms = sm_count();
+    export_fused_kernel<<<ntiles < sms ? ntiles : sms, kXThreads, smem, s>>>(tmap, a);
     LE_LAUNCHED();
     return LE_OK;
 }

@@ -48,6 +48,22 @@ def test_feature_map(leg, orc, P, ncb, d):
     assert e2 <= 2e-2
 
 
+@pytest.mark.parametrize("P,ncb,d", [(20000, 48, 320), (20000, 176, 128), (129, 144, 64), (40000, 32, 896)])
+def test_feature_map_odd_units(leg, P, ncb, d):
+    """Code counts whose 16-code units split unevenly over a tile's two warpgroups or leave a short last
+    codebook block, odd multiples of 64 dims, one and two tiles per slot."""
+    import paper_2311_18482_gb300 as L
+    dec = synth.decoder_init(43, ncb)
+    feat, _, _ = _inputs(P, ncb, 44)
+    S = np.random.default_rng(45).standard_normal((ncb, d)).astype(np.float32)
+    F = L.le_feature_map(_t(feat), _dec_t(dec), _t(S))
+    L.le_device_status()
+    z = emulate_logits(feat, dec)
+    e = np.exp(z - z.max(0))
+    emu = bf16(((bf16(e).T @ bf16(S)) / e.sum(0)[:, None]))
+    assert fro(F.to(torch.float32).cpu().numpy().astype(np.float64), emu) <= 3e-3
+
+
 def test_feature_map_one_hot(leg, orc):
     """A decoder whose logits single out one code by a wide margin: F is that code's BF16 row."""
     import paper_2311_18482_gb300 as L
