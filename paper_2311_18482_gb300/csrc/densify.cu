@@ -260,7 +260,8 @@ __device__ __forceinline__ void child_rows(const ScatterArgs& a, size_t base, co
 // copy bound by HBM: at 1M Gaussians of SH degree 3 (900k left, 1.13M out) it
 // reads and writes 1.7 GB.  One thread per Gaussian walking its own rows
 // touched 32 rows per warp instruction (the whole call took 0.733 ms); rows
-// dealt out by output unit make every warp access consecutive (0.333 ms).
+// dealt out by output unit make every warp access consecutive (0.333 ms).  While
+// all blocks are resident anyway, each field has blocks of its own.
 template <int NC>
 __global__ void __launch_bounds__(256) densify_scatter_kernel(ScatterArgs a)
 {
@@ -305,21 +306,30 @@ __global__ void __launch_bounds__(256) densify_scatter_kernel(ScatterArgs a)
     const Segment clone = {list[1], (int)run[1], K1 + a.boff[(size_t)a.nb + cb] + skip[1]};
     const Segment split = {list[2], (int)run[2], K1 + K2 + 2 * (size_t)(a.boff[2 * (size_t)a.nb + cb] + skip[2])};
     // a field moves in 16-byte units when its rows are whole multiples of them and its six arrays are aligned
-    copy_rows<float, 3>(a, 0, base, kept, clone, split);
-    copy_rows<float, 3>(a, 1, base, kept, clone, split);
-    if (a.vec & 4u) copy_rows<float4, 1>(a, 2, base, kept, clone, split);
-    else copy_rows<float, 4>(a, 2, base, kept, clone, split);
-    copy_rows<float, 1>(a, 3, base, kept, clone, split);
-    if constexpr (3 * NC % 4 == 0) {
-        if (a.vec & 16u) copy_rows<float4, 3 * NC / 4>(a, 4, base, kept, clone, split);
-        else copy_rows<float, 3 * NC>(a, 4, base, kept, clone, split);
-    } else {
-        copy_rows<float, 3 * NC>(a, 4, base, kept, clone, split);
+    const auto mine = [](int f) { return gridDim.y == 1 || (int)blockIdx.y == f; };
+    if (mine(0)) {
+        copy_rows<float, 3>(a, 0, base, kept, clone, split);
+        child_rows(a, base, split);
     }
-    if (a.vec & 32u) copy_rows<float4, 2>(a, 5, base, kept, clone, split);
-    else copy_rows<float, 8>(a, 5, base, kept, clone, split);
-    copy_rows<float, 1>(a, 6, base, kept, clone, split);
-    child_rows(a, base, split);
+    if (mine(1)) copy_rows<float, 3>(a, 1, base, kept, clone, split);
+    if (mine(2)) {
+        if (a.vec & 4u) copy_rows<float4, 1>(a, 2, base, kept, clone, split);
+        else copy_rows<float, 4>(a, 2, base, kept, clone, split);
+    }
+    if (mine(3)) copy_rows<float, 1>(a, 3, base, kept, clone, split);
+    if (mine(4)) {
+        if constexpr (3 * NC % 4 == 0) {
+            if (a.vec & 16u) copy_rows<float4, 3 * NC / 4>(a, 4, base, kept, clone, split);
+            else copy_rows<float, 3 * NC>(a, 4, base, kept, clone, split);
+        } else {
+            copy_rows<float, 3 * NC>(a, 4, base, kept, clone, split);
+        }
+    }
+    if (mine(5)) {
+        if (a.vec & 32u) copy_rows<float4, 2>(a, 5, base, kept, clone, split);
+        else copy_rows<float, 8>(a, 5, base, kept, clone, split);
+    }
+    if (mine(6)) copy_rows<float, 1>(a, 6, base, kept, clone, split);
 }
 
 Fields fields_of(const le_gaussian_grads* g)
@@ -456,7 +466,9 @@ extern "C" le_status le_densify(const le_densify_config* cfg, const le_gaussians
         if (aligned16(a.p.f[i]) && aligned16(a.m.f[i]) && aligned16(a.v.f[i]) && aligned16(a.po.f[i]) &&
             aligned16(a.mo.f[i]) && aligned16(a.vo.f[i]))
             a.vec |= 1u << i;
-    const int sb = (n + kSB - 1) / kSB;
+    // up to here seven blocks per 512 Gaussians are resident at once (152 SMs x 8 blocks)
+    const int blocks = (n + kSB - 1) / kSB;
+    const dim3 sb(blocks, 7 * blocks <= 152 * 8 ? 7 : 1);
     switch (g->sh_degree) {
         case 0: densify_scatter_kernel<1><<<sb, 256, 0, s>>>(a); break;
         case 1: densify_scatter_kernel<4><<<sb, 256, 0, s>>>(a); break;
