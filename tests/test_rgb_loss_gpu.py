@@ -28,6 +28,19 @@ def test_rgb_loss(leg, orc, W, H, lam):
     assert np.all(np.abs(got - o["loss"]) <= 1e-5 * np.abs(o["loss"]))
 
 
+@pytest.mark.parametrize("W,H", [(1, 1), (31, 33), (64, 32), (65, 97), (32, 11)])
+def test_rgb_loss_tile_edges(leg, orc, W, H):
+    """Images smaller than a tile, exact multiples of it and one pixel more: loss 1e-5, gradient 1e-4."""
+    rng = np.random.default_rng(W * 100 + H)
+    img = rng.uniform(0, 1, (3, H, W)).astype(np.float32)
+    tgt = rng.uniform(0, 1, (3, H, W)).astype(np.float32)
+    loss, grad = leg.le_rgb_loss(torch.from_numpy(img).cuda(), torch.from_numpy(tgt).cuda(), lambda_ssim=0.2)
+    torch.cuda.synchronize()
+    o = orc.rgb_loss(img, tgt, lam=0.2)
+    assert rel_err(grad.cpu().numpy(), o["grad"]) < 1e-4
+    assert np.all(np.abs(loss.cpu().numpy().astype(np.float64) - o["loss"]) <= 1e-5 * np.abs(o["loss"]))
+
+
 def test_training_step_with_dssim(leg):
     """A few training steps with 3DGS's full RGB loss lower it on a fixed view."""
     from paper_2311_18482_gb300.training import TrainState
