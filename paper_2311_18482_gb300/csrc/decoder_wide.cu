@@ -382,11 +382,16 @@ __global__ void __launch_bounds__(kThreads, 1) wide_kernel(WideArgs a)
                         add_bias16(v, b3s + c);
                     }
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        v[j] = c < ncb ? g * (__expf(v[j] - lse) - (c + j == t ? 1.f : 0.f)) : 0.f;
+                    for (int j = 0; j < 16; ++j) v[j] = c < ncb ? g * __expf(v[j] - lse) : 0.f;
                     uint32_t w[8];
                     pack16(v, w);
                     store_cols<TRAIN, 128>(sA, blob + kBZ, row, c, w);
+                }
+                if (t >= zc0 && t < zc1) {          // the target's column once more, with its -1
+                    const __nv_bfloat16 b = __float2bfloat16_rn(g * (__expf(zt - lse) - 1.f));
+                    const uint32_t o = sbuf_off(row, t, 128);
+                    *reinterpret_cast<__nv_bfloat16*>(sA + o) = b;
+                    *reinterpret_cast<__nv_bfloat16*>(blob + kBZ + o) = b;
                 }
             }
         }
