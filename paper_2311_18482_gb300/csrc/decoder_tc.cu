@@ -5,7 +5,7 @@
 // 128-pixel tile: the rendered feature R_s of the tile is the A operand of
 // three chained MMAs whose accumulators never leave the SM; the CUDA cores
 // only apply bias + ReLU between layers (TMEM -> registers -> BF16 shared
-// memory) and the softmax at the end.  Three kernels share that front end:
+// memory) and the softmax at the end.  Four kernels share that front end:
 //
 //   dec_fwd_kernel    inference (supp. Sec. "Inference"): argmax and/or
 //                     M_infer = softmax(logits), two tiles in flight per CTA.
@@ -24,9 +24,8 @@
 //                     p^T (S_c S_c^T) p and phi.q_j = p.(S_c q_j)/|F_clip|; the
 //                     relevancy does not depend on the scale of p, so neither
 //                     the softmax normaliser nor the 896-dim feature map F is
-//                     ever formed; S_c S_c^T (N x N) is streamed through shared
-//                     memory in 64-column chunks with 1-D bulk async copies,
-//                     S_c [q; n] sits in shared memory.
+//                     ever formed.
+//   export_fused_kernel the feature map F itself, where a consumer wants it.
 //
 // Every mbarrier wait is bounded (about a second); on timeout the kernel
 // records it in g_tc_error, stops issuing work, frees its TMEM and returns.
@@ -52,15 +51,13 @@ struct DecArgs {
     float *dW1, *db1, *dW2, *db2, *dW3, *db3;
     int32_t* argmax;
     float* prob;
-    // query: W3 as its BF16 shared-memory image
-    const unsigned char* W3_img;
+    // query and feature-map export: the back phase's operand, a chunked BF16 image
+    // (query_prep_kernel, codebook_chunks_kernel) of `dd` rows or dims
+    const unsigned char* G_img;
+    int dd;
     // query
-    const unsigned char* G_img;     // ncb/64 chunks of [ncb x 64] canonical bf16
-    const float* Aq;                // [16, ncb] fp32 = [text; negs] S_c^T
     int Q, n_neg;
     float* rel;
-    // feature-map export
-    int dd;                         // feature dims d (multiple of 64)
     // training with the RGB L1 term of the same pixels (nullable img): img, img_t [3, P],
     // d_img [3, P] = sign(img - img_t) inv_l1, *loss_l1 += sum |img - img_t| inv_l1
     const float *img, *img_t;
@@ -84,11 +81,6 @@ struct Front {
     bool issuer;       // the warp that issues this group's MMAs (warp-uniform)
     int half, nhalf;
     float4* xch;       // [nhalf][128] (nhalf > 1 only)
-    // W3s reloaded by a bulk copy (the issuing warp): the third layer's MMAs wait
-    // for it first
-    uint64_t* w3bar = nullptr;
-    uint32_t w3phase = 0;
-    bool w3pending = false;
 };
 
 // Columns [c0, c1) of an N-column epilogue handled by this thread's half (units of 16).
@@ -176,19 +168,12 @@ __device__ bool mlp_forward_x(Front& f, const DecArgs& a, const float* x)
         sts_row16(smem_u32(f.H2.p) + sbuf_off(f.tid, c, f.H2.C), w);
     }
     wg_publish(f);
-    if (f.issuer) {
-        if (f.w3pending) {
-            if (!mbar_wait(f.w3bar, f.w3phase)) atomicExch(&g_tc_error, 1);
-            f.w3phase ^= 1u;
-            f.w3pending = false;
-        }
-        if (elect_one()) {
-            const uint32_t id = idesc_bf16(a.ncb, false, false);
+    if (f.issuer && elect_one()) {
+        const uint32_t id = idesc_bf16(a.ncb, false, false);
 #pragma unroll
-            for (int s = 0; s < kH2 / 16; ++s)
-                mma(f.tw, kdesc(f.H2, 0, 16 * s), kdesc(f.W3s, 0, 16 * s), id, s > 0);
-            commit(f.mbar);
-        }
+        for (int s = 0; s < kH2 / 16; ++s)
+            mma(f.tw, kdesc(f.H2, 0, 16 * s), kdesc(f.W3s, 0, 16 * s), id, s > 0);
+        commit(f.mbar);
     }
     return wg_wait(f);
 }
@@ -255,7 +240,6 @@ __device__ unsigned char* load_weights(unsigned char* base, const DecArgs& a, Fr
 // 128 codes in flight and a branch per logit in the softmax, 10,000 / 300,000 /
 // 1,088,640 pixels took 19.8 / 114 / 370 us at 128 codes and 31.8 / 194 / 629 us
 // at 256; now 10.3 / 52 / 157 us and 14.7 / 100 / 322 us.
-constexpr size_t kFwdWgBytes = sbuf_bytes(128, 16) + sbuf_bytes(128, 64) + sbuf_bytes(128, 128);
 constexpr size_t kFwdTileBytes = sbuf_bytes(128, 128);
 
 __host__ constexpr size_t fwd_smem(int ncb, int nwg) { return weights_bytes(ncb) + nwg * kFwdTileBytes + 128; }
@@ -820,241 +804,35 @@ __global__ void __launch_bounds__(kTrainThreads, 1) dec_train_kernel(DecArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// Query: decode, softmax (unnormalised), relevancy.  Four warpgroups per CTA serve the same
-// 128 rows and split every epilogue by columns; TMEM: logits in [0, ncb)
-// (later the 16 text/negative projections in [0, 16) and the four parts'
-// partial p^T G p in columns 16-19), p^T G in [256, 256 + ncb).  The
-// activations X1/H1/H2, the parts' softmax exchange and the BF16 softmax P
-// share one region (each is written after the last reader of the previous
-// one has finished).
-constexpr uint32_t kTG = 256;
-constexpr int kQueryParts = 4;
-
-__host__ constexpr size_t query_smem(int ncb)
-{
-    return weights_bytes(ncb) + sbuf_bytes(16, ncb) +
-           (sbuf_bytes(128, ncb) > kFwdWgBytes ? sbuf_bytes(128, ncb) : kFwdWgBytes) + 2 * sbuf_bytes(ncb, 64) + 128;
-}
-
-__global__ void __launch_bounds__(128 * kQueryParts, 1) query_fused_kernel(DecArgs a)
-{
-    extern __shared__ __align__(1024) unsigned char sm[];
-    Front f;
-    unsigned char* p = load_weights(sm, a, f);
-    const SBuf Aqs{p, a.ncb};
-    p += sbuf_bytes(16, a.ncb);
-    f.X1 = SBuf{p, 16};
-    f.H1 = SBuf{p + sbuf_bytes(128, 16), 64};
-    f.H2 = SBuf{p + sbuf_bytes(128, 16) + sbuf_bytes(128, 64), 128};
-    const SBuf Ps{p, a.ncb};
-    f.xch = reinterpret_cast<float4*>(p);
-    p += sbuf_bytes(128, a.ncb) > kFwdWgBytes ? sbuf_bytes(128, a.ncb) : kFwdWgBytes;
-    // G in 64-column chunks: chunks 0 and 1 stay in their own slots for the whole
-    // kernel; chunks 2 and 3 (n_cb > 128) go into W3's shared memory, which
-    // holds exactly two chunks and is idle from the end of the third layer's
-    // MMAs to the next tile's: they are copied in while the softmax runs, and
-    // W3 is copied back (from its global image) while the relevancy and the
-    // next tile's first two layers run, so no copy is on the tile's path.
-    const uint32_t chunk_bytes = sbuf_bytes(a.ncb, 64);
-    unsigned char* const g_own = p;
-    auto g_chunk = [&](int kc) {
-        return SBuf{kc < 2 ? g_own + kc * chunk_bytes : f.W3s.p + (kc - 2) * chunk_bytes, 64};
-    };
-    p += 2 * chunk_bytes;
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(p);     // [0] MMA, [1] chunks 0-1, [2] chunks 2-3, [4] W3
-    uint32_t* slot = reinterpret_cast<uint32_t*>(p + 24);
-    const int tid = threadIdx.x;
-    sbuf_fill(Aqs, 16, a.Aq, a.ncb, 16, a.ncb);
-    f.mbar = mbar;
-    f.phase = 0;
-    f.tid = tid & 127;
-    f.bar_id = 0;
-    f.nthreads = blockDim.x;
-    const int warp = (int)warp_uniform(threadIdx.x >> 5);
-    f.half = warp >> 2;
-    f.issuer = warp == 0;
-    f.nhalf = kQueryParts;
-    f.w3bar = mbar + 4;
-    if (tid == 0) {
-        for (int i = 0; i < 3; ++i) mbar_init(mbar + i, 1);
-        mbar_init(mbar + 4, 1);
-    }
-    if (tid < 32) tmem_alloc(slot, 512);
-    fence_proxy_async();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(slot));
-    f.tw = tbase;
-    f.lane = (uint32_t)(32 * ((tid >> 5) & 3)) << 16;
-    const int row = f.tid;
-    int c0, c1;
-    my_cols(f, a.ncb, c0, c1);                  // this part's class columns
-    const int nch = a.ncb / 64;                 // G chunks (64 K-columns each)
-    const int nlow = nch < 2 ? nch : 2, nup = nch - nlow;
-    // loads in flight (the issuing warp): chunks 0-1 (once), chunks 2-3 (per tile)
-    bool low_pending = false, up_pending = false;
-    uint32_t up_phase = 0u;
-    const int ntiles = (a.P + 127) / 128;
-    bool ok = true;
-    if (f.issuer && (int)blockIdx.x < ntiles) {
-        if (elect_one()) {
-            mbar_expect_tx(mbar + 1, nlow * chunk_bytes);
-            bulk_g2s(g_own, a.G_img, nlow * chunk_bytes, mbar + 1);
-        }
-        low_pending = true;
-    }
-    float xf[8];                                // this tile's R_s, loaded a tile ahead (part 0)
-    if (f.half == 0) load_feat(a, blockIdx.x * 128 + row, blockIdx.x * 128 + row < a.P, xf);
-    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int px = tile * 128 + row;
-        const bool valid = px < a.P;
-        if (!mlp_forward_x(f, a, xf)) break;
-        // the third layer's MMAs have read W3: chunks 2-3 of G take its place
-        if (f.issuer && nup > 0) {
-            if (elect_one()) {
-                mbar_expect_tx(mbar + 2, nup * chunk_bytes);
-                bulk_g2s(f.W3s.p, a.G_img + 2 * (size_t)chunk_bytes, nup * chunk_bytes, mbar + 2);
-            }
-            up_pending = true;
-        }
-        if (f.half == 0) {
-            const int nx = px + 128 * (int)gridDim.x;
-            load_feat(a, nx, tile + (int)gridDim.x < ntiles && nx < a.P, xf);
-        }
-        // e = exp(z - max z) in BF16.  The relevancy phi.q / |phi| with
-        // phi = sum_c p_c s_c does not depend on the scale of p, so the
-        // softmax normaliser 1 / sum e is never needed.
-        float v[16], mh = -INFINITY;
-        for (int c = c0; c < c1; c += 16) {
-            tmem_ld16(f.tw + f.lane + c, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) mh = fmaxf(mh, v[j] + f.b3s[c + j]);
-        }
-        f.xch[f.half * 128 + row].x = mh;
-        wg_sync(f);
-        float m = -INFINITY;
-#pragma unroll
-        for (int h = 0; h < kQueryParts; ++h) m = fmaxf(m, f.xch[h * 128 + row].x);
-        wg_sync(f);
-        const float ml = m * 1.4426950408889634f;
-        for (int c = c0; c < c1; c += 16) {
-            tmem_ld16(f.tw + f.lane + c, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = ex2_approx(fmaf(v[j] + f.b3s[c + j], 1.4426950408889634f, -ml));
-            sbuf_store8(Ps, row, c, v);
-            sbuf_store8(Ps, row, c + 8, v + 8);
-        }
-        wg_publish(f);
-        // p . (S_c [q; n]) into [0, 16), p^T G into [256, 256 + ncb), all chunks in one round
-        bool tmo = false;
-        if (f.issuer) {
-            const uint64_t pd = kdesc(Ps, 0, 0), qd = kdesc(Aqs, 0, 0);
-            const uint32_t id = idesc_bf16(a.ncb, false, false);
-            for (int kc = 0; kc < nch; ++kc)
-                if (elect_one())
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        mma(tbase, pd + 64 * kc + 16 * k, qd + 64 * kc + 16 * k, idesc_bf16(16, false, false),
-                            kc > 0 || k > 0);
-            if (low_pending) {
-                if (!mbar_wait(mbar + 1, 0u)) tmo = true;
-                low_pending = false;
-            }
-            for (int kc = 0; kc < nch; ++kc) {
-                if (kc == 2) {
-                    if (!mbar_wait(mbar + 2, up_phase)) tmo = true;
-                    up_phase ^= 1u;
-                    up_pending = false;
-                }
-                const uint64_t gd = kdesc(g_chunk(kc), 0, 0);
-                if (elect_one())
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        mma(tbase + kTG, pd + 64 * kc + 16 * k, gd + 16 * k, id, kc > 0 || k > 0);
-            }
-            if (elect_one()) commit(f.mbar);
-        }
-        if (!wg_wait(f) || bar_any(0, blockDim.x, tmo)) {
-            if (tid == 0) atomicExch(&g_tc_error, 1);
-            break;
-        }
-        // the G MMAs are done with W3's shared memory: W3 goes back for the next tile
-        if (f.issuer && nup > 0 && tile + (int)gridDim.x < ntiles) {
-            if (elect_one()) {
-                mbar_expect_tx(f.w3bar, sbuf_bytes(a.ncb, 128));
-                bulk_g2s(f.W3s.p, a.W3_img, sbuf_bytes(a.ncb, 128), f.w3bar);
-            }
-            f.w3pending = true;
-        }
-        // relevancy: each part sums e^T G e over its columns into TMEM column 16 + part
-        float ptgp = 0.f, pp[16];
-        for (int c = c0; c < c1; c += 16) {
-            tmem_ld16(tbase + kTG + f.lane + c, v);
-            sbuf_load8(Ps, row, c, pp);
-            sbuf_load8(Ps, row, c + 8, pp + 8);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) ptgp = fmaf(pp[j], v[j], ptgp);
-        }
-        tmem_st1(tbase + f.lane + 16 + f.half, ptgp);
-        tmem_wait_st();
-        fence_before();
-        __syncthreads();
-        fence_after();
-        if (f.half == 0) {
-            tmem_ld16(tbase + f.lane, v);        // the 16 projections and the parts' partial sums
-            float tot = 0.f, w[16];
-            tmem_ld16(tbase + f.lane + 16, w);
-#pragma unroll
-            for (int h = 0; h < kQueryParts; ++h) tot += w[h];
-            const float inv = rsqrtf(fmaxf(tot, 1e-30f));
-            // unrolled with constant indices: v stays in registers (a runtime
-            // index would put it, and every TMEM load into it, in local memory)
-            float smax = -INFINITY;
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (j >= a.Q && j < a.Q + a.n_neg) smax = fmaxf(smax, v[j] * inv);
-            if (valid)
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    if (j < a.Q) a.rel[(size_t)j * a.P + px] = 1.f / (1.f + __expf(smax - v[j] * inv));
-        }
-        fence_before();
-        __syncthreads();
-    }
-    // drain copies still in flight (only after an early exit) before the shared memory goes away
-    if (f.issuer) {
-        if (low_pending) mbar_wait(mbar + 1, 0u);
-        if (up_pending) mbar_wait(mbar + 2, up_phase);
-        if (f.w3pending) mbar_wait(f.w3bar, f.w3phase);
-    }
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (tid < 32) tmem_dealloc(tbase, 512);
-}
-
-// ---------------------------------------------------------------------------
-// Language feature map export F = M_infer S (supp. Sec. "Inference"): per
-// pixel the decoder's softmax p over the n_cb codes times the codebook, in
-// BF16; e = exp(z - max z) is rounded to BF16 and each output row is scaled by
-// 1 / sum e.  Two 128-pixel tiles are in flight per CTA, each with its own two
-// warpgroups, MMA warp and load warp, going through two phases:
+// Query (relevancy) and language feature map export, both a decode followed by a
+// contraction of the tile's softmax numerators e = exp(z - max z), in BF16, with
+// a constant operand B:
+//   export  F = M_infer S (supp. Sec. "Inference"): B = the codebook S, each
+//           output row scaled by 1 / sum e, BF16 out;
+//   query   B = [ [text; negs] S_c^T | S_c S_c^T ]: the projections e.(S_c q) and
+//           e^T G, from which |phi|^2 = e^T G e (relevancy does not depend on
+//           the scale of e, so its sum is never needed).
+// Two 128-pixel tiles are in flight per CTA, each with its own two warpgroups,
+// MMA warp and load warp, going through two phases:
 //   front  the warpgroups decode the tile and write e over its logits in tensor
 //          memory, as the A operand of
-//   back   F = e S in 128-dim chunks.  The codebook streams through the tile's
-//          four 8 KB slots ([32 codes x 128 dims], bulk copies), the MMA warp
-//          contracts them into 128 TMEM columns, and the warpgroups drain a
-//          finished chunk, 64 dims each, through two 64-byte-swizzled staging
-//          boxes and TMA tensor stores (128 pixels x 32 dims).
+//   back   e B in 128-column chunks.  B streams through the tile's four 8 KB
+//          slots ([32 codes x 128 columns], bulk copies), the MMA warp contracts
+//          them into 128 TMEM columns, and the warpgroups drain a finished
+//          chunk, 64 columns each: the export through two 64-byte-swizzled
+//          staging boxes and TMA tensor stores (128 pixels x 32 dims), the query
+//          into its running e^T G e.
 // The second tile starts when the first one enters its back phase, so one tile's
 // front, bound by the latency of its rounds, runs beside the other's MMAs and
 // stores.  e in tensor memory leaves shared memory for the slots; N = 128 because
-// an MMA of N = 64 takes three quarters as long.  A 1296 x 840 view at 256 codes:
-// 0.679 ms (2.9 TB/s written); two tiles in phase sharing every slot 0.812 ms, the
-// same with e in shared memory 0.886 ms, one tile at a time in rounds of two
-// 64-dim chunks 1.255 ms.  Per tile, 45,000 cycles: 17,000 in the front, 13,000
-// waiting for the codebook (the latency of four slots), 13,000 of MMAs.
+// an MMA of N = 64 takes three quarters as long.  Export of a 1296 x 840 view at
+// 256 codes: 0.679 ms (2.9 TB/s written); two tiles in phase sharing every slot
+// 0.812 ms, the same with e in shared memory 0.886 ms, one tile at a time in rounds
+// of two 64-dim chunks 1.255 ms.  Per tile, 45,000 cycles: 17,000 in the front,
+// 13,000 waiting for the codebook (the latency of four slots), 13,000 of MMAs.
+// A query of 2,073,600 pixels against 256 codes takes 0.730 ms, of 72,261 against
+// 64 codes 37 us (0.863 ms and 43 us with one tile at a time, four warpgroups on it
+// and G partly resident in shared memory).
 constexpr int kXSlots = 4, kXCodes = 32, kXDims = 128;
 constexpr uint32_t kXSlotBytes = sbuf_bytes(kXCodes, kXDims), kXBox = sbuf_bytes(128, 32);
 // A tile's region: X1 and H1, then H2 over them; in the back phase two staging boxes per warpgroup.
@@ -1077,8 +855,8 @@ __host__ constexpr size_t export_smem(int ncb)
 }
 static_assert(export_smem(256) <= 227 * 1024 && 2 * sizeof(ExportBars) + 4 <= 256, "export shared memory");
 
-__global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid_constant__ CUtensorMap tmap_out,
-                                                                    DecArgs a)
+template <bool QUERY>
+__device__ __forceinline__ void decode_contract(const CUtensorMap* tmap_out, const DecArgs& a)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char* const act =
@@ -1112,7 +890,7 @@ __global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid
     const uint32_t tbase = warp_uniform(*reinterpret_cast<volatile uint32_t*>(tslot));
     const int ntiles = (a.P + 127) / 128;
     const int nch = (a.dd + kXDims - 1) / kXDims, nkb = (ncb + kXCodes - 1) / kXCodes;
-    const auto width = [&](int j) { return min(kXDims, a.dd - j * kXDims); };        // 128, or 64 in the last chunk
+    const auto width = [&](int j) { return min(kXDims, a.dd - j * kXDims); };        // 128, or less in the last chunk
     const auto codes = [&](int k) { return min(kXCodes, ncb - k * kXCodes); };       // 32, or 16 in the last block
     // tile slot t takes the tiles blockIdx.x + gridDim.x (t + 2 i)
     const int t = warp < 16 ? warp >> 3 : warp & 1;
@@ -1123,7 +901,7 @@ __global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid
     bool ok = true;
 
     if (warp >= 18) {
-        // the codebook, chunk by chunk, for every tile of the slot
+        // B, chunk by chunk, for every tile of the slot
         uint32_t it = 0;
         for (int tile = first; tile < ntiles && ok; tile += stride)
             for (int j = 0; j < nch && ok; ++j) {
@@ -1152,19 +930,21 @@ __global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid
         for (int tile = first; tile < ntiles && ok; tile += stride, ++r) {
             if (!(ok = warp_agree(mbar_wait(&bar->e_ready, r & 1u)))) break;
             for (int j = 0; j < nch && ok; ++j, ++c) {
-                const uint32_t C = (uint32_t)width(j), id = idesc_bf16((int)C, false, true);
+                const uint32_t C = (uint32_t)width(j), id = idesc_bf16((int)C, false, !QUERY);
                 if (c >= 1 && !(ok = warp_agree(mbar_wait(&bar->acc_free, (c - 1) & 1u)))) break;
                 fence_after();
                 for (int k = 0; k < nkb; ++k, ++it) {
                     const uint32_t sl = it % kXSlots;
                     if (!(ok = warp_agree(mbar_wait(bar->full + sl, (it / kXSlots) & 1u)))) break;
                     fence_after();
-                    const uint64_t gm = mndesc_at(slots_a + sl * kXSlotBytes, (int)C, 0, 0);
+                    // export: rows are codes (K), read MN-major; query: rows are columns of B (N)
+                    const uint32_t at = slots_a + sl * kXSlotBytes;
+                    const uint64_t gm = QUERY ? kdesc_at(at, kXCodes, 0, 0) : mndesc_at(at, (int)C, 0, 0);
                     const uint32_t ea = td + 8u * (kXCodes / 16) * k;
                     const bool two = codes(k) > 16;
                     if (elect_one()) {
                         mma_ta(td + kXAcc, ea, gm, id, k > 0);
-                        if (two) mma_ta(td + kXAcc, ea + 8u, gm + 2ull * C, id, 1u);
+                        if (two) mma_ta(td + kXAcc, ea + 8u, gm + (QUERY ? 16ull : 2ull * C), id, 1u);
                         commit(bar->empty + sl);
                         if (k + 1 == nkb) commit(&bar->acc_full);
                     }
@@ -1260,13 +1040,16 @@ __global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid
                     if (i < held) tmem_st8(tl + 8 * (hu + i), hold[i]);
             }
             tmem_wait_st();
-            sums[wg * 128 + row] = se;
+            if (!QUERY) sums[wg * 128 + row] = se;
             fence_before();
             wg_sync(f);
             fence_after();
             if (lead && f.half == 0) mbar_arrive(&bar->e_ready);
-            const float inv = valid ? 1.0f / (sums[2 * t * 128 + row] + sums[(2 * t + 1) * 128 + row]) : 0.f;
+            const float inv = !QUERY && valid ? 1.0f / (sums[2 * t * 128 + row] + sums[(2 * t + 1) * 128 + row]) : 0.f;
+            float pj[16], quad = 0.f;               // query: the projections (half 0), e^T G e over this half's columns
             for (int j = 0; j < nch; ++j, ++c) {
+                // the next tile's R_s while the last chunk's MMAs run (the export has no registers to spare here)
+                if (QUERY && j + 1 == nch && f.half == 0) load_feat(a, nx, more, xf);
                 const bool got = mbar_wait(&bar->acc_full, c & 1u);
                 // every thread of the tile leaves together
                 if (bar_any(f.bar_id, 256, !got)) {
@@ -1274,46 +1057,91 @@ __global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid
                     break;
                 }
                 fence_after();
-                const bool mine = 64 * f.half < width(j);
-                __nv_bfloat162 h[32];
-                if (mine) {
+                if constexpr (QUERY) {
+                    // 16-column units of the chunk: unit 0 of the first chunk holds the projections, the others
+                    // columns of G in order
+                    const int w16 = width(j) / 16, wh = (w16 + 1) / 2;
+                    for (int u = f.half ? wh : 0; u < (f.half ? w16 : wh); ++u) {
+                        tmem_ld16(tl + kXAcc + 16 * u, v);
+                        const int col = 8 * j + u - 1;      // unit of G
+                        if (col < 0) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        tmem_ld16(tl + kXAcc + 64u * f.half + 16u * q, v);
+                            for (int i = 0; i < 16; ++i) pj[i] = v[i];
+                            continue;
+                        }
+                        tmem_ld8(tl + 8 * col, w);
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            h[8 * q + i] = __floats2bfloat162_rn(v[2 * i] * inv, v[2 * i + 1] * inv);
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 e2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(w + i));
+                            quad = fmaf(e2.x, v[2 * i], quad);
+                            quad = fmaf(e2.y, v[2 * i + 1], quad);
+                        }
                     }
-                }
-                fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bar->acc_free);
-                if (!mine) continue;
-                // row-major 64-byte rows, 16-byte unit u of row r at u ^ ((r >> 1) & 3); a box is rewritten once
-                // the store before the last one has read it
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar->acc_free);
+                } else {
+                    const bool mine = 64 * f.half < width(j);
+                    __nv_bfloat162 h[32];
+                    if (mine) {
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    if (lead) bulk_wait_read_but_one();
-                    asm volatile("bar.sync %0, 128;" ::"r"(3 + wg) : "memory");
+                        for (int q = 0; q < 4; ++q) {
+                            tmem_ld16(tl + kXAcc + 64u * f.half + 16u * q, v);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        *reinterpret_cast<uint4*>(stg + q * kXBox + row * 64 + ((u ^ ((row >> 1) & 3)) << 4)) =
-                            *reinterpret_cast<uint4*>(h + 16 * q + 4 * u);
-                    fence_proxy_async();
-                    asm volatile("bar.sync %0, 128;" ::"r"(3 + wg) : "memory");
-                    if (lead) {
-                        tma_store_2d(&tmap_out, kXDims * j + 64 * f.half + 32 * q, tile * 128, stg + q * kXBox);
-                        bulk_commit();
+                            for (int i = 0; i < 8; ++i)
+                                h[8 * q + i] = __floats2bfloat162_rn(v[2 * i] * inv, v[2 * i + 1] * inv);
+                        }
+                    }
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar->acc_free);
+                    if (!mine) continue;
+                    // row-major 64-byte rows, 16-byte unit u of row r at u ^ ((r >> 1) & 3); a box is rewritten once
+                    // the store before the last one has read it
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        if (lead) bulk_wait_read_but_one();
+                        asm volatile("bar.sync %0, 128;" ::"r"(3 + wg) : "memory");
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            *reinterpret_cast<uint4*>(stg + q * kXBox + row * 64 + ((u ^ ((row >> 1) & 3)) << 4)) =
+                                *reinterpret_cast<uint4*>(h + 16 * q + 4 * u);
+                        fence_proxy_async();
+                        asm volatile("bar.sync %0, 128;" ::"r"(3 + wg) : "memory");
+                        if (lead) {
+                            tma_store_2d(tmap_out, kXDims * j + 64 * f.half + 32 * q, tile * 128, stg + q * kXBox);
+                            bulk_commit();
+                        }
                     }
                 }
             }
             if (!ok) break;
+            if constexpr (QUERY) {
+                // the halves' sums meet in shared memory; phi.q / |phi| from the projections
+                if (f.half) sums[wg * 128 + row] = quad;
+                fence_before();
+                wg_sync(f);
+                fence_after();
+                if (!f.half) {
+                    const float inv = rsqrtf(fmaxf(quad + sums[(wg + 1) * 128 + row], 1e-30f));
+                    float smax = -INFINITY;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (i >= a.Q && i < a.Q + a.n_neg) smax = fmaxf(smax, pj[i] * inv);
+                    if (valid)
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (i < a.Q)
+                                a.rel[(size_t)i * a.P + tile * 128 + row] = 1.f / (1.f + __expf(smax - pj[i] * inv));
+                }
+                continue;
+            }
             if (f.half == 0) load_feat(a, nx, more, xf);
             // the next tile's X1 and H1 go where the staging boxes are
             if (lead) bulk_wait_read_all();
             wg_sync(f);
         }
-        if (lead) bulk_wait_all();
+        if (!QUERY && lead) bulk_wait_all();
     }
     fence_before();
     const bool bad = __syncthreads_or(!ok);
@@ -1322,17 +1150,13 @@ __global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid
     if (warp == 0) tmem_dealloc(tbase, 512);
 }
 
-// W3 [ncb x 128] (fp32) -> its BF16 shared-memory image (the layout load_weights writes).
-__global__ void w3_image_kernel(const float* __restrict__ W3, int ncb, unsigned char* __restrict__ img)
+__global__ void __launch_bounds__(kXThreads, 1) export_fused_kernel(const __grid_constant__ CUtensorMap tmap_out,
+                                                                    DecArgs a)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncb * (kH2 / 8); i += gridDim.x * blockDim.x) {
-        const int r = i / (kH2 / 8), c0 = (i % (kH2 / 8)) * 8;
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = W3[(size_t)r * kH2 + c0 + j];
-        sbuf_store8(SBuf{img, kH2}, r, c0, v);
-    }
+    decode_contract<false>(&tmap_out, a);
 }
+
+__global__ void __launch_bounds__(kXThreads, 1) query_fused_kernel(DecArgs a) { decode_contract<true>(nullptr, a); }
 
 // The export's codebook S [ncb x dd] (fp32) as a chunked canonical BF16 image:
 // chunk j holds dims [128 j, 128 j + 128) (64 in the last chunk of an odd multiple
@@ -1351,21 +1175,20 @@ __global__ void codebook_chunks_kernel(const float* __restrict__ S, int ncb, int
     }
 }
 
-// Query constants in one launch, 16 x 16 outputs per block, k ascending with
-// FMAs (the order of a plain dot product):
-//   block rows y < ncb/16:  G = S_c S_c^T, written straight into its chunked
-//                           canonical BF16 image: chunk kc holds columns
-//                           [64 kc, 64 kc + 64) of every row as an [ncb x 64]
-//                           canonical buffer;
-//   block row y = ncb/16:   Aq[r][j] = [text; negs]_r . S_c[j] (rows r >= Q + n_neg zero).
+// The query's operand B in one launch, 16 x 16 entries per block, k ascending with
+// FMAs (the order of a plain dot product), as a chunked BF16 image: chunk j holds
+// rows [128 j, 128 j + 128) of
+//   rows 0 - 15:     [text; negs] S_c^T (rows past Q + n_neg zero)
+//   rows 16 - ...:   G = S_c S_c^T
+// in blocks of 32 codes, each an [rows x 32] canonical buffer.
 __global__ void __launch_bounds__(256) query_prep_kernel(const float* __restrict__ S, int ncb, int dd, int d_clip,
                                                          const float* __restrict__ text, int Q,
                                                          const float* __restrict__ negs, int n_neg,
-                                                         unsigned char* __restrict__ img, float* __restrict__ Aq)
+                                                         unsigned char* __restrict__ img)
 {
     __shared__ float xs[16][33], ys[16][33];
-    const int j0 = blockIdx.x * 16, i0 = blockIdx.y * 16;
-    const bool gram = i0 < ncb;
+    const int j0 = blockIdx.x * 16, i0 = ((int)blockIdx.y - 1) * 16;
+    const bool gram = i0 >= 0;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     float acc = 0.f;
     for (int k0 = 0; k0 < d_clip; k0 += 32) {
@@ -1385,15 +1208,9 @@ __global__ void __launch_bounds__(256) query_prep_kernel(const float* __restrict
         for (int c = 0; c < 32; ++c) acc = fmaf(xs[ty][c], ys[tx][c], acc);
         __syncthreads();
     }
-    const int r = i0 + ty, c = j0 + tx;
-    if (gram) {
-        const int kc = c >> 6, cc = c & 63;
-        unsigned char* dst = img + (size_t)kc * ncb * 64 * 2 + ((r >> 3) * 8 * 128 + (cc >> 3) * 128 + (r & 7) * 16) +
-                             (cc & 7) * 2;
-        *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(acc);
-    } else {
-        Aq[(size_t)ty * ncb + c] = acc;
-    }
+    const int r = i0 + 16 + ty, c = j0 + tx, j = r / kXDims, rows = min(kXDims, 16 + ncb - j * kXDims);
+    unsigned char* blk = img + (size_t)j * kXDims * ncb * 2 + (size_t)(c / kXCodes) * rows * kXCodes * 2;
+    *reinterpret_cast<__nv_bfloat16*>(blk + sbuf_off(r - j * kXDims, c % kXCodes, kXCodes)) = __float2bfloat16_rn(acc);
 }
 
 // Self-test of the bounded-wait path: waits on an mbarrier that nothing ever
@@ -1502,7 +1319,7 @@ le_status decode_fused(int32_t P, const float* feat, const float* unc, const le_
     return LE_OK;
 }
 
-// W3's BF16 shared-memory image [n_cb x 128], Aq [16 x n_cb] FP32, G's BF16 image [n_cb x n_cb].
+// The image of the query's operand takes 2 (n_cb + 16) n_cb bytes of this.
 size_t query_fused_workspace(int32_t, int32_t n_cb, int32_t)
 {
     return align_up(256ull * n_cb, 256) + align_up(sizeof(float) * 16 * n_cb, 256) + align_up(2ull * n_cb * n_cb, 256);
@@ -1519,36 +1336,24 @@ le_status query_fused(int32_t P, const float* feat, const le_decoder* d, const f
         set_error("fused query needs n_cb to be a multiple of 64 (got %d)", ncb);
         return LE_ERR_UNSUPPORTED;
     }
-    char* w = static_cast<char*>(ws);
-    unsigned char* w3img = reinterpret_cast<unsigned char*>(w);
-    float* Aq = reinterpret_cast<float*>(w + align_up(256ull * ncb, 256));
-    unsigned char* img = reinterpret_cast<unsigned char*>(w + align_up(256ull * ncb, 256) +
-                                                          align_up(sizeof(float) * 16 * ncb, 256));
-    // G = S_c S_c^T (as the BF16 image) and Aq = [text; negs] S_c^T, FP32 on CUDA cores, one launch
+    unsigned char* img = static_cast<unsigned char*>(ws);
     query_prep_kernel<<<dim3(ncb / 16, ncb / 16 + 1), 256, 0, s>>>(codebook, ncb, dd, d_clip, text, Q, negs, n_neg,
-                                                                   img, Aq);
+                                                                   img);
     LE_LAUNCHED();
-    // W3's shared-memory image, reloaded after each tile when G's chunks 2-3 borrow its place (n_cb > 128)
-    if (ncb > 128) {
-        w3_image_kernel<<<16, 256, 0, s>>>(d->W3, ncb, w3img);
-        LE_LAUNCHED();
-    }
     DecArgs a{};
     a.P = P;
     a.ncb = ncb;
     a.feat = feat;
     a.W1 = d->W1; a.b1 = d->b1; a.W2 = d->W2; a.b2 = d->b2; a.W3 = d->W3; a.b3 = d->b3;
     a.G_img = img;
-    a.W3_img = w3img;
-    a.Aq = Aq;
+    a.dd = 16 + ncb;
     a.Q = Q;
     a.n_neg = n_neg;
     a.rel = rel;
-    const size_t smem = query_smem(ncb);
+    const size_t smem = export_smem(ncb);
     if ((st = set_smem(query_fused_kernel, smem)) != LE_OK) return st;
-    const int ntiles = (P + 127) / 128;
-    const int grid = ntiles < sm_count() ? ntiles : sm_count();
-    query_fused_kernel<<<grid, 128 * kQueryParts, smem, s>>>(a);
+    const int ntiles = (P + 127) / 128, sms = sm_count();
+    query_fused_kernel<<<ntiles < sms ? ntiles : sms, kXThreads, smem, s>>>(a);
     LE_LAUNCHED();
     return LE_OK;
 }

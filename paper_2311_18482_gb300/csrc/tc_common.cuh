@@ -186,6 +186,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// 8 consecutive words of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r)
+{
+    asm volatile(
+        "{\ntcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+        "tcgen05.wait::ld.sync.aligned;\n}\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr)
+        : "memory");
+}
+
 // Store 16 FP32 values to consecutive columns of this thread's TMEM lane; call
 // tmem_wait_st() before reading them back.
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v)
