@@ -42,7 +42,13 @@ constexpr int kStages = 5;
 constexpr int kRows = 128;           // features per tile (MMA M)
 constexpr int kChunk = 64;           // BF16 columns per stage (one 128-byte swizzle span)
 constexpr uint32_t kATile = kRows * kChunk * 2;
-constexpr int kThreads = 448;
+// Warps: TMA producer, MMA issuer, four for the feature norms, and kParts(GRAD)
+// epilogue warps per TMEM lane quadrant, which split a row's columns.  The
+// gradient's epilogue (two passes of about 25 instructions a value) bounds that
+// kernel, so it has four per quadrant: le_quantize_grad on 300,007 features takes
+// 0.295 ms, 0.341 with two, scalar table reads and a two-byte store per value.
+__host__ __device__ constexpr int parts_of(bool grad) { return grad ? 4 : 2; }
+__host__ __device__ constexpr int threads_of(bool grad) { return 32 * (6 + 4 * parts_of(grad)); }
 // Every CTA reads the whole BF16 codebook once per tile from L2.  To keep 152
 // SMs from hammering the same L2 lines at the same moment, the prep kernel
 // writes kCopies copies (CTA b reads copy b % kCopies) and each CTA walks the
@@ -92,21 +98,23 @@ struct Smem {
     uint32_t bstride;
     uint64_t *full, *empty, *acc_full, *acc_empty, *norm_ready, *norm_free, *fin;
     float* norms;                // [2 slots][2][128] inverse feature norms
-    float* xch;                  // [2 slots][2 halves][4][128] epilogue exchange
+    float* xch;                  // [2 slots][parts][4][128] epilogue exchange
     float* rv;                   // [N] utilisation ratio (gradient mode)
     float* inv_s;                // [2][N]
     unsigned* cnt;               // [N]
     uint32_t* tmem_slot;
 };
 
-__host__ __device__ constexpr uint32_t quant_smem_bytes(int N)
+__host__ __device__ constexpr uint32_t xch_bytes(bool grad) { return 2 * 4 * parts_of(grad) * kRows * 4; }
+
+__host__ __device__ constexpr uint32_t quant_smem_bytes(int N, bool grad)
 {
-    return 1024 + kStages * (kATile + (uint32_t)N * kChunk * 2) + 2 * 2 * kRows * 4 + 2 * 8 * kRows * 4 + N * 4 +
+    return 1024 + kStages * (kATile + (uint32_t)N * kChunk * 2) + 2 * 2 * kRows * 4 + xch_bytes(grad) + N * 4 +
            2 * N * 4 + N * 4 + 8 +
            (2 * kStages + 10) * 8;
 }
 
-__device__ Smem carve(unsigned char* base, int N)
+__device__ Smem carve(unsigned char* base, int N, bool grad)
 {
     Smem s;
     unsigned char* p = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(base) + 1023) & ~uintptr_t(1023));
@@ -118,7 +126,7 @@ __device__ Smem carve(unsigned char* base, int N)
     s.norms = reinterpret_cast<float*>(p);
     p += 2 * 2 * kRows * 4;
     s.xch = reinterpret_cast<float*>(p);
-    p += 2 * 8 * kRows * 4;
+    p += xch_bytes(grad);
     s.rv = reinterpret_cast<float*>(p);
     p += N * 4;
     s.inv_s = reinterpret_cast<float*>(p);
@@ -185,6 +193,25 @@ __device__ __forceinline__ float warp_colsum16(float* v, int lane)
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
+__device__ __forceinline__ void load4(const float* p, float* v)
+{
+    const float4 u = *reinterpret_cast<const float4*>(p);
+    v[0] = u.x;
+    v[1] = u.y;
+    v[2] = u.z;
+    v[3] = u.w;
+}
+
+// Two lanes' (rows r, r + 1) values a, b of codes j, j + 1 as two BF16 pairs, one
+// per lane: the even lane stores code j's at p (its own p), the odd lane code
+// j + 1's.  A row past the end (have = false) contributes 0 to its pair's other row.
+__device__ __forceinline__ void store_pair(__nv_bfloat16* p, float a, float b, bool odd, bool have, bool store)
+{
+    const float mine = have ? (odd ? b : a) : 0.f, send = have ? (odd ? a : b) : 0.f;
+    const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
+    if (store) *reinterpret_cast<__nv_bfloat162*>(p) = odd ? __floats2bfloat162_rn(recv, mine) : __floats2bfloat162_rn(mine, recv);
+}
+
 // The i-th chunk this CTA processes within a tile: the CLIP chunks [0, nclip)
 // first, then the DINO chunks, each part rotated by the CTA's offset.
 __device__ __forceinline__ int chunk_at(int i, int nclip, int nchunks, int rot)
@@ -194,13 +221,14 @@ __device__ __forceinline__ int chunk_at(int i, int nclip, int nchunks, int rot)
 }
 
 template <bool GRAD>
-__global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constant__ CUtensorMap tmap_f,
+__global__ void __launch_bounds__(threads_of(GRAD), 1) quant_kernel(const __grid_constant__ CUtensorMap tmap_f,
                                                             const __grid_constant__ CUtensorMap tmap_s, QuantArgs q)
 {
     extern __shared__ unsigned char smem_raw[];
     const int N = q.N;
-    Smem s = carve(smem_raw, N);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int NP = parts_of(GRAD);
+    Smem s = carve(smem_raw, N, GRAD);
+    const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) s.inv_s[i] = q.inv_s[i];
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         s.cnt[i] = 0u;
@@ -213,9 +241,9 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(s.acc_full + i, 1);
-            mbar_init(s.acc_empty + i, 2 * kRows);
+            mbar_init(s.acc_empty + i, NP * kRows);
             mbar_init(s.norm_ready + i, kRows);
-            mbar_init(s.norm_free + i, 2 * kRows);
+            mbar_init(s.norm_free + i, NP * kRows);
         }
         mbar_init(s.fin, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -226,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(s.tmem_slot);
+    const uint32_t tmem = warp_uniform(*reinterpret_cast<volatile uint32_t*>(s.tmem_slot));
     const uint32_t b_bytes = (uint32_t)N * kChunk * 2;
     bool ok = true;
 
@@ -264,8 +292,11 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
+        // ---------------- MMA issuer: the whole warp (the index map of 1.09M features 0.373 -> 0.361 ms), but one
+        // lane in gradient mode, where the epilogue bounds the kernel and the waits of a whole warp cost 2 %
+        const auto agree = [](bool got) { return GRAD ? got : warp_agree(got); };
+        const auto lead = [] { return GRAD || elect_one(); };
+        if (!GRAD || lane == 0) {
             const uint32_t idesc = idesc_bf16(N, false, false);
             int st = 0;
             uint32_t ph = 0;
@@ -273,14 +304,14 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
             for (int t = blockIdx.x; t < q.ntiles && ok; t += gridDim.x, ++it) {
                 const int slot = it & 1;
                 const uint32_t aph = (uint32_t)(it >> 1) & 1u;
-                if (!wait_bar(s.acc_empty + slot, aph ^ 1)) {
+                if (!agree(wait_bar(s.acc_empty + slot, aph ^ 1))) {
                     ok = false;
                     break;
                 }
                 fence_after();
                 const uint32_t acc = tmem + (uint32_t)(2 * N * slot);
                 for (int c = 0; c < q.nchunks; ++c) {
-                    if (!wait_bar(s.full + st, ph)) {
+                    if (!agree(wait_bar(s.full + st, ph))) {
                         ok = false;
                         break;
                     }
@@ -289,21 +320,22 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
                     const uint32_t d = acc + (clip ? 0u : (uint32_t)N);
                     const uint64_t da = desc_sw128(smem_u32(s.a0 + st * kATile)),
                                    db = desc_sw128(smem_u32(s.b0 + st * s.bstride));
+                    const uint32_t keep = (c != 0 && c != q.nclip) ? 1u : 0u;
+                    if (lead()) {
 #pragma unroll
-                    for (int k = 0; k < kChunk / 16; ++k) {
-                        const uint32_t accumulate = (k > 0 || (c != 0 && c != q.nclip)) ? 1u : 0u;
-                        mma(d, da + 2u * k, db + 2u * k, idesc, accumulate);
+                        for (int k = 0; k < kChunk / 16; ++k) mma(d, da + 2u * k, db + 2u * k, idesc, k > 0 ? 1u : keep);
+                        commit(s.empty + st);
                     }
-                    commit(s.empty + st);
+                    if (!GRAD) __syncwarp();
                     if (++st == kStages) {
                         st = 0;
                         ph ^= 1;
                     }
                 }
                 if (!ok) break;
-                commit(s.acc_full + slot);
+                if (lead()) commit(s.acc_full + slot);
             }
-            commit(s.fin);
+            if (lead()) commit(s.fin);
             (void)wait_bar(s.fin, 0);      // every MMA of ours has completed
         }
     } else if (warp < 6) {
@@ -354,25 +386,26 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
             mbar_arrive(s.norm_ready + slot);
         }
     } else {
-        // ---------------- epilogue: row = TMEM lane 32 (warp % 4) + lane; half h of the
-        // 16-column chunks (h = 0: chunks [0, nh0), h = 1: [nh0, N/16))
+        // ---------------- epilogue: row = TMEM lane 32 (warp % 4) + lane; part h of the
+        // 16-column chunks
         const int quad = warp & 3, h = (warp - 6) >> 2;
         const int r = 32 * quad + lane;
         const uint32_t lanef = (uint32_t)(32 * quad) << 16;
-        const int nch = N / 16, nh0 = (nch + 1) / 2;
-        const int c_lo = h ? nh0 : 0, c_hi = h ? nch : nh0;
-        float psum[4], usum[4];   // softmax column sums (gradient mode: sums of g cos^C, g cos^D)
+        constexpr int kPC = 8 / NP;               // chunks of a part at N = 128
+        const int nch = N / 16, per = (nch + NP - 1) / NP;
+        const int c_lo = min(nch, h * per), c_hi = min(nch, (h + 1) * per);
+        float psum[kPC], usum[kPC];   // softmax column sums (gradient mode: sums of g cos^C, g cos^D)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) psum[i] = usum[i] = 0.f;
+        for (int i = 0; i < kPC; ++i) psum[i] = usum[i] = 0.f;
         float lcos = 0.f;
         int it = 0;
         for (int t = blockIdx.x; t < q.ntiles && ok; t += gridDim.x, ++it) {
             const int slot = it & 1;
             const uint32_t aph = (uint32_t)(it >> 1) & 1u;
-            // the two warps of a quadrant decide together, so that a timeout never
+            // the warps of a quadrant decide together, so that a timeout never
             // leaves one of them at the exchange barrier below
             const bool got = wait_bar(s.norm_ready + slot, aph) && wait_bar(s.acc_full + slot, aph);
-            if (bar_any(1 + quad, 64, !got)) {
+            if (bar_any(1 + quad, 32 * NP, !got)) {
                 ok = false;
                 break;
             }
@@ -394,53 +427,81 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
                     tmem_ld16(acc + j0, vc);
                     tmem_ld16(acc + N + j0, vd);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float dv = fmaf(vc[k] * aC, s.inv_s[j0 + k], vd[k] * aD * s.inv_s[N + j0 + k]);
-                        if (dv > best) {
-                            best = dv;
-                            bi = j0 + k;
+                    for (int k4 = 0; k4 < 16; k4 += 4) {
+                        float ic[4], id[4], rv[4];
+                        load4(s.inv_s + j0 + k4, ic);
+                        load4(s.inv_s + N + j0 + k4, id);
+                        load4(s.rv + j0 + k4, rv);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float dv = fmaf(vc[k4 + k] * aC, ic[k], vd[k4 + k] * aD * id[k]);
+                            if (dv > best) {
+                                best = dv;
+                                bi = j0 + k4 + k;
+                            }
+                            const float e = __expf(dv);
+                            esum += e;
+                            esr = fmaf(e, rv[k], esr);
                         }
-                        const float e = __expf(dv);
-                        esum += e;
-                        esr = fmaf(e, s.rv[j0 + k], esr);
                     }
                 }
-                float* x = s.xch + slot * 8 * kRows;
+                float* x = s.xch + slot * 4 * NP * kRows;
                 x[(4 * h) * kRows + r] = best;
                 x[(4 * h + 1) * kRows + r] = __int_as_float(bi);
                 x[(4 * h + 2) * kRows + r] = esum;
                 x[(4 * h + 3) * kRows + r] = esr;
-                named_sync(1 + quad, 64);
-                const float ob = x[(4 * (1 - h)) * kRows + r];
-                const int oi = __float_as_int(x[(4 * (1 - h) + 1) * kRows + r]);
-                esum += x[(4 * (1 - h) + 2) * kRows + r];
-                esr += x[(4 * (1 - h) + 3) * kRows + r];
-                if (h == 0 ? ob > best : ob >= best) bi = oi;
+                named_sync(1 + quad, 32 * NP);
+                best = -INFINITY;
+                bi = 0;
+                esum = esr = 0.f;
+#pragma unroll
+                for (int o = 0; o < NP; ++o) {          // ties: the lower part, the lower indices
+                    const float ob = x[(4 * o) * kRows + r];
+                    if (ob > best) {
+                        best = ob;
+                        bi = __float_as_int(x[(4 * o + 1) * kRows + r]);
+                    }
+                    esum += x[(4 * o + 2) * kRows + r];
+                    esr += x[(4 * o + 3) * kRows + r];
+                }
                 const float inv_e = valid ? 1.0f / esum : 0.f;
                 const float sigma = esr * inv_e;
                 // pass 2: g_ij = lambda_lb/K s_ij (r_j - sigma_i) - lambda_cos/K [j = m_i];
-                // u^C_j += g cos^C_ij, u^D_j += g cos^D_ij; G^T scaled by the inverse feature norms
+                // u^C_j += g cos^C_ij, u^D_j += g cos^D_ij; G^T scaled by the inverse feature norms, the rows of a
+                // lane pair side by side (the even lane stores code j's two, the odd lane code j + 1's)
+                const bool odd = lane & 1;
+                const bool store = (row & ~1ll) < q.K;
 #pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
+                for (int cc = 0; cc < kPC; ++cc) {
                     const int c = c_lo + cc;
                     if (c >= c_hi) break;
                     const int j0 = 16 * c;
                     float vc[16], vd[16];
                     tmem_ld16(acc + j0, vc);
                     tmem_ld16(acc + N + j0, vd);
+                    const size_t at = (size_t)(j0 + odd) * q.kp + (row & ~1ll);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float cosc = vc[k] * aC0 * s.inv_s[j0 + k], cosd = vd[k] * aD0 * s.inv_s[N + j0 + k];
-                        const float sv = __expf(fmaf(q.lambda_d, cosd, cosc)) * inv_e;
-                        float g = q.cl * sv * (s.rv[j0 + k] - sigma);
-                        if (j0 + k == bi) g -= q.cc;
-                        g = valid ? g : 0.f;
-                        if (valid) {
-                            q.gtc[(size_t)(j0 + k) * q.kp + row] = __float2bfloat16_rn(g * aC0);
-                            q.gtd[(size_t)(j0 + k) * q.kp + row] = __float2bfloat16_rn(g * aD0);
+                    for (int k4 = 0; k4 < 16; k4 += 4) {
+                        float ic[4], id[4], rv[4], g[4];
+                        load4(s.inv_s + j0 + k4, ic);
+                        load4(s.inv_s + N + j0 + k4, id);
+                        load4(s.rv + j0 + k4, rv);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float cosc = vc[k4 + k] * aC0 * ic[k], cosd = vd[k4 + k] * aD0 * id[k];
+                            const float sv = __expf(fmaf(q.lambda_d, cosd, cosc)) * inv_e;
+                            g[k] = q.cl * sv * (rv[k] - sigma);
+                            if (j0 + k4 + k == bi) g[k] -= q.cc;
+                            g[k] = valid ? g[k] : 0.f;
+                            vc[k4 + k] = valid ? g[k] * cosc : 0.f;     // rows past K: cos is NaN
+                            vd[k4 + k] = valid ? g[k] * cosd : 0.f;
                         }
-                        vc[k] = valid ? g * cosc : 0.f;     // rows past K: cos is NaN
-                        vd[k] = valid ? g * cosd : 0.f;
+#pragma unroll
+                        for (int k = 0; k < 4; k += 2) {
+                            const size_t o = at + (size_t)(k4 + k) * q.kp;
+                            store_pair(q.gtc + o, g[k] * aC0, g[k + 1] * aC0, odd, store && valid, store);
+                            store_pair(q.gtd + o, g[k] * aD0, g[k + 1] * aD0, odd, store && valid, store);
+                        }
                     }
                     psum[cc] += warp_colsum16(vc, lane);
                     usum[cc] += warp_colsum16(vd, lane);
@@ -459,14 +520,20 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
                     tmem_ld16(acc + j0, vc);
                     tmem_ld16(acc + N + j0, vd);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float dv = fmaf(vc[k] * aC, s.inv_s[j0 + k], vd[k] * aD * s.inv_s[N + j0 + k]);
-                        if (dv > best) {
-                            best = dv;
-                            bi = j0 + k;
+                    for (int k4 = 0; k4 < 16; k4 += 4) {
+                        float ic[4], id[4];
+                        load4(s.inv_s + j0 + k4, ic);
+                        load4(s.inv_s + N + j0 + k4, id);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float dv = fmaf(vc[k4 + k] * aC, ic[k], vd[k4 + k] * aD * id[k]);
+                            if (dv > best) {
+                                best = dv;
+                                bi = j0 + k4 + k;
+                            }
+                            vc[k4 + k] = __expf(dv);
+                            esum += vc[k4 + k];
                         }
-                        vc[k] = __expf(dv);
-                        esum += vc[k];
                     }
                     tmem_st16(acc + j0, vc);
                 }
@@ -475,7 +542,7 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
                 x[(3 * h) * kRows + r] = best;
                 x[(3 * h + 1) * kRows + r] = __int_as_float(bi);
                 x[(3 * h + 2) * kRows + r] = esum;
-                named_sync(1 + quad, 64);
+                named_sync(1 + quad, 32 * NP);
                 const float ob = x[(3 * (1 - h)) * kRows + r];
                 const int oi = __float_as_int(x[(3 * (1 - h) + 1) * kRows + r]);
                 esum += x[(3 * (1 - h) + 2) * kRows + r];
@@ -487,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
                 tmem_wait_st();
                 // pass 2: softmax column sums of this half's columns over the warp's 32 rows
 #pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
+                for (int cc = 0; cc < kPC; ++cc) {
                     const int c = c_lo + cc;
                     if (c >= c_hi) break;
                     float e[16];
@@ -512,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
             if (GRAD) {
                 if ((lane & 1) == 0)
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc)
+                    for (int cc = 0; cc < kPC; ++cc)
                         if (c_lo + cc < c_hi) {
                             atomicAdd(q.u + 16 * (c_lo + cc) + (lane >> 1), psum[cc]);
                             atomicAdd(q.u + N + 16 * (c_lo + cc) + (lane >> 1), usum[cc]);
@@ -521,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1) quant_kernel(const __grid_constan
                 if (lane == 0 && h == 0) atomicAdd(q.lcos, lcos);
                 if ((lane & 1) == 0)
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc)
+                    for (int cc = 0; cc < kPC; ++cc)
                         if (c_lo + cc < c_hi) atomicAdd(q.psum + 16 * (c_lo + cc) + (lane >> 1), psum[cc]);
             }
         }
@@ -882,10 +949,10 @@ extern "C" le_status le_quantize(int64_t K, int32_t d, int32_t d_clip, const uin
     q.psum = w.psum;
     q.count = w.count;
     q.lcos = w.lcos;
-    const uint32_t smem = quant_smem_bytes(n_cb);
+    const uint32_t smem = quant_smem_bytes(n_cb, false);
     LE_CUDA(cudaFuncSetAttribute(quant_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int grid = q.ntiles < sms ? q.ntiles : sms;
-    quant_kernel<false><<<grid, kThreads, smem, s>>>(mf, ms, q);
+    quant_kernel<false><<<grid, threads_of(false), smem, s>>>(mf, ms, q);
     LE_LAUNCHED();
     quant_finalize_kernel<<<1, 128, 0, s>>>(w.psum, w.count, w.lcos, n_cb, K, lambda_cos, lambda_lb, r, p, loss);
     LE_LAUNCHED();
@@ -990,10 +1057,10 @@ extern "C" le_status le_quantize_grad(int64_t K, int32_t d, int32_t d_clip, cons
     q.u = w.u;
     q.cl = lambda_lb / (float)K;
     q.cc = lambda_cos / (float)K;
-    const uint32_t smem = quant_smem_bytes(n_cb);
+    const uint32_t smem = quant_smem_bytes(n_cb, true);
     LE_CUDA(cudaFuncSetAttribute(quant_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int grid = q.ntiles < sms ? q.ntiles : sms;
-    quant_kernel<true><<<grid, kThreads, smem, s>>>(mf, ms, q);
+    quant_kernel<true><<<grid, threads_of(true), smem, s>>>(mf, ms, q);
     LE_LAUNCHED();
     GemmArgs ga;
     ga.N = n_cb;
