@@ -166,7 +166,7 @@ le_status exclusive_scan(In in, int n, uint32_t* out, uint32_t* partials, uint32
 // ----------------------------------------------------------------------------
 // Depth sort: stable LSD radix sort of e = bits(depth) << 32 | index on bits
 // 32-63 in four 8-bit passes.  Each pass is count / scan / scatter over tiles
-// of kSortTile consecutive elements, and no block waits on another:
+// of 512 ITEMS consecutive elements, and no block waits on another:
 //   count    per-tile digit counts, counts[d][b] (digit-major, rows padded to
 //            a multiple of 4), and the digits' totals (pass 0's are counted
 //            while the keys are built);
@@ -179,9 +179,17 @@ le_status exclusive_scan(In in, int n, uint32_t* out, uint32_t* partials, uint32
 // into depth order (zero for culled Gaussians) for the kernels that follow.
 constexpr int kSortPasses = 4;
 constexpr int kSortThreads = 512;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;   // 4096 elements per tile
+constexpr int kSortItems = 8;                          // the largest tile: 4096 elements
+constexpr int kSortTile = kSortThreads * kSortItems;
 constexpr int kSortWarps = kSortThreads / 32;
+
+// Elements per thread of a pass.  Few Gaussians want small tiles: a pass takes as
+// long as one tile does while every tile has an SM of its own.  le_bin_sort with
+// tiles of 1,024 / 2,048 / 4,096 elements: 100,000 Gaussians 138 / 148 / 176 us,
+// 400,000 152 / 158 / 180, 600,000 203 / 193 / 202, 1M 269 / 255 / 266, 3M 638 /
+// 583 / 591.  The largest tiles remain for counts whose digit table would not fit
+// where the smaller ones' lies (from 134M).
+inline int sort_items(int n) { return n <= 450000 ? 2 : (n <= 1 << 26 ? 4 : kSortItems); }
 
 __device__ __forceinline__ uint32_t digit_of(uint64_t e, int shift) { return (uint32_t)(e >> shift) & 255u; }
 
@@ -199,6 +207,7 @@ __device__ __forceinline__ void publish_counts(const uint32_t* h, uint32_t* coun
 }
 
 // e[i] (culled: 0xFFFFFFFF in the high word, sorted last) and pass 0's counts.
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) depth_elems_kernel(int n, const float* __restrict__ depth,
                                                                    const int* __restrict__ tiles,
                                                                    uint64_t* __restrict__ e, uint32_t* counts,
@@ -208,8 +217,8 @@ __global__ void __launch_bounds__(kSortThreads) depth_elems_kernel(int n, const 
     if (threadIdx.x < 256) h[threadIdx.x] = 0;
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) {
-        const int i = blockIdx.x * kSortTile + k * kSortThreads + threadIdx.x;
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = blockIdx.x * (kSortThreads * ITEMS) + k * kSortThreads + threadIdx.x;
         if (i < n) {
             const uint32_t hi = tiles[i] > 0 ? __float_as_uint(depth[i]) : 0xFFFFFFFFu;
             e[i] = ((uint64_t)hi << 32) | (uint32_t)i;
@@ -221,6 +230,7 @@ __global__ void __launch_bounds__(kSortThreads) depth_elems_kernel(int n, const 
 }
 
 // Per-tile counts of the digit (e >> shift) & 255.
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const uint64_t* __restrict__ in, int n, int shift,
                                                                   uint32_t* counts, int row, uint32_t* totals)
 {
@@ -228,8 +238,8 @@ __global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const uint64_t
     if (threadIdx.x < 256) h[threadIdx.x] = 0;
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) {
-        const int i = blockIdx.x * kSortTile + k * kSortThreads + threadIdx.x;
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = blockIdx.x * (kSortThreads * ITEMS) + k * kSortThreads + threadIdx.x;
         if (i < n) atomicAdd(&h[digit_of(in[i], shift)], 1u);
     }
     __syncthreads();
@@ -290,12 +300,14 @@ struct SortGather {
 
 // One pass on digit (e >> shift) & 255 from in to out; offsets: counts after
 // sort_rowscan_kernel.  gather.drect non-null: also gather into depth order.
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64_t* __restrict__ in,
                                                                     uint64_t* __restrict__ out, int n, int shift,
                                                                     const uint32_t* __restrict__ offsets, int row,
                                                                     SortGather gather)
 {
-    __shared__ uint64_t stage[kSortTile];
+    constexpr int kTileElems = kSortThreads * ITEMS;
+    __shared__ uint64_t stage[kTileElems];
     __shared__ uint32_t warp_cnt[kSortWarps][256];
     __shared__ uint32_t gbase[256], lbase[256];
     __shared__ uint32_t ws[kSortWarps];
@@ -303,22 +315,22 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64
     for (int j = threadIdx.x; j < kSortWarps * 256; j += kSortThreads) (&warp_cnt[0][0])[j] = 0;
     if (threadIdx.x < 256) gbase[threadIdx.x] = offsets[(size_t)threadIdx.x * row + blockIdx.x];
     __syncthreads();
-    const int base = blockIdx.x * kSortTile;
-    const int cnt = min(kSortTile, n - base);
+    const int base = blockIdx.x * kTileElems;
+    const int cnt = min(kTileElems, n - base);
 
     // each warp owns the contiguous sub-range [w * 256, (w + 1) * 256) of the tile
     const uint32_t lt = (1u << lane) - 1u;
-    uint64_t e[kSortItems];
-    uint32_t dg[kSortItems];
+    uint64_t e[ITEMS];
+    uint32_t dg[ITEMS];
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) {
-        const int j = w * (kSortTile / kSortWarps) + k * 32 + lane;
+    for (int k = 0; k < ITEMS; ++k) {
+        const int j = w * (kTileElems / kSortWarps) + k * 32 + lane;
         const bool valid = j < cnt;
         e[k] = valid ? in[base + j] : 0ull;
         dg[k] = valid ? digit_of(e[k], shift) : 0xFFFFFFFFu;
     }
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
         const uint32_t vm = __ballot_sync(0xffffffffu, dg[k] != 0xFFFFFFFFu);
         if (dg[k] != 0xFFFFFFFFu) {
             const uint32_t peers = __match_any_sync(vm, dg[k]);
@@ -343,7 +355,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64
     __syncthreads();
     // stage the tile's elements in digit order (stable), then write them out
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
         const bool valid = dg[k] != 0xFFFFFFFFu;
         const uint32_t vm = __ballot_sync(0xffffffffu, valid);
         uint32_t peers = 0, pos = 0;
@@ -721,7 +733,7 @@ __host__ __device__ constexpr size_t seg(size_t bytes) { return (bytes + 255) / 
 // The depth sort's digit totals, [passes][256].
 __host__ __device__ constexpr size_t sort_state_words(int) { return (size_t)kSortPasses * 256; }
 
-// The depth sort's per-tile counts / offsets, [256][sort_row(n)].
+// The depth sort's counts / offsets of the largest tiles, [256][sort_row(n)].
 __host__ __device__ constexpr size_t sort_count_words(int n) { return 256ull * sort_row(n); }
 
 // Scratch layout of le_bin_sort for n Gaussians (independent of the copy count).
@@ -758,23 +770,30 @@ SortWs sort_ws_layout(char* base, int32_t n)
     return w;
 }
 
-// The four passes (pass 0's counts are in w.counts and w.sort_state, counted
-// by depth_elems_kernel).  Result in *cur; the rectangles and tile ellipses in
-// depth order in w.drect and w.dell.
-le_status depth_sort(uint64_t*& cur, uint64_t*& alt, int n, const SortWs& w, const SortGather& gather, cudaStream_t s)
+// The depth sort: keys and pass 0's counts, then the four passes.  Result in cur
+// (alt: the other buffer); the rectangles and tile ellipses in depth order in
+// w.drect and w.dell.  Smaller tiles' digit counts lie in w.base, which the copy
+// counts take over afterwards (128 bytes per Gaussian; the smallest tiles need 1).
+template <int ITEMS>
+le_status depth_sort(uint64_t*& cur, uint64_t*& alt, int n, const SortWs& w, const float* depth,
+                     const SortGather& gather, cudaStream_t s)
 {
-    const int nt = sort_tiles(n), row = sort_row(n);
+    const int nt = (n + kSortThreads * ITEMS - 1) / (kSortThreads * ITEMS), row = (nt + 3) / 4 * 4;
+    uint32_t* const counts = ITEMS == kSortItems ? w.counts : w.base;
+    LE_CUDA(cudaMemsetAsync(w.sort_state, 0, 4 * sort_state_words(n), s));
+    depth_elems_kernel<ITEMS><<<nt, kSortThreads, 0, s>>>(n, depth, gather.tiles, cur, counts, row, w.sort_state);
+    LE_LAUNCHED();
     for (int q = 0; q < kSortPasses; ++q) {
         const int shift = 32 + 8 * q;
         uint32_t* totals = w.sort_state + 256 * q;
         if (q > 0) {
-            sort_count_kernel<<<nt, kSortThreads, 0, s>>>(cur, n, shift, w.counts, row, totals);
+            sort_count_kernel<ITEMS><<<nt, kSortThreads, 0, s>>>(cur, n, shift, counts, row, totals);
             LE_LAUNCHED();
         }
-        sort_rowscan_kernel<<<256 / 8, 256, 0, s>>>(w.counts, nt, row, totals);
+        sort_rowscan_kernel<<<256 / 8, 256, 0, s>>>(counts, nt, row, totals);
         LE_LAUNCHED();
-        sort_scatter_kernel<<<nt, kSortThreads, 0, s>>>(cur, alt, n, shift, w.counts, row,
-                                                        q == kSortPasses - 1 ? gather : SortGather{});
+        sort_scatter_kernel<ITEMS><<<nt, kSortThreads, 0, s>>>(cur, alt, n, shift, counts, row,
+                                                               q == kSortPasses - 1 ? gather : SortGather{});
         LE_LAUNCHED();
         uint64_t* t = cur;
         cur = alt;
@@ -844,12 +863,12 @@ le_status bin_prepare(const le_camera* cam, int32_t n, const float* depth, const
         depth_rank_kernel<<<(n + kElems - 1) / kElems, kRankThreads, 0, s>>>(n, depth, cur, gather);
         LE_LAUNCHED();
     } else {
-        LE_CUDA(cudaMemsetAsync(w.sort_state, 0, 4 * sort_state_words(n), s));
-        depth_elems_kernel<<<sort_tiles(n), kSortThreads, 0, s>>>(n, depth, tiles_touched, w.eA, w.counts, sort_row(n),
-                                                                  w.sort_state);
-        LE_LAUNCHED();
         uint64_t* alt = w.eB;
-        if ((st = depth_sort(cur, alt, n, w, gather, s)) != LE_OK) return st;
+        const int items = sort_items(n);
+        st = items == 8   ? depth_sort<8>(cur, alt, n, w, depth, gather, s)
+             : items == 4 ? depth_sort<4>(cur, alt, n, w, depth, gather, s)
+                          : depth_sort<2>(cur, alt, n, w, depth, gather, s);
+        if (st != LE_OK) return st;
     }
     // copies per (tile, chunk of depth-sorted Gaussians)
     const size_t diff_smem = sizeof(int4) * (((size_t)(TX + 1) * TY + 3) / 4);

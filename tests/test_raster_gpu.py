@@ -185,6 +185,27 @@ def test_binning_order_on_both_sorts(leg, orc, n):
     assert np.array_equal(ranges.cpu().numpy().view(np.uint32).reshape(-1), np.asarray(ref["ranges"]).reshape(-1))
 
 
+@pytest.mark.parametrize("n", [100_003, 450_000, 450_001, 1_000_003])
+def test_depth_order_on_both_tiles(leg, n):
+    """Both tile sizes of the radix sort: on one column of tiles, every list is in (depth, index) order."""
+    rng = np.random.default_rng(n)
+    c = synth.config("c1", n=4, W=16, H=16)
+    cam = c["camera"]
+    depth = torch.from_numpy(rng.choice(rng.uniform(0.5, 9.0, n // 3).astype(np.float32), n)).cuda()
+    proj = leg.Projected.empty(n)
+    proj.depth.copy_(depth)
+    seen = torch.from_numpy((rng.uniform(size=n) < 0.02).astype(np.int32)).cuda()
+    proj.tiles_touched.copy_(seen)
+    proj.rect.copy_(torch.tensor([0, 0, 1, 1], dtype=torch.int16).cuda().expand(n, 4) * seen[:, None].to(torch.int16))
+    # an ellipse that reaches the whole tile: centred on it, a long way wide and high
+    proj.tile_ellipse.copy_(torch.tensor([8.0, 8.0, 0.0, 1.0, 1e6, 0.0, 0.25, 0.25]).cuda().expand(n, 8))
+    ids, ranges, K, _ = leg.le_bin_sort(cam, proj)
+    idx = torch.nonzero(seen).view(-1)
+    order = torch.sort(depth[idx], stable=True)[1]
+    assert K == len(idx)
+    assert torch.equal(ids.long(), idx[order])
+
+
 def test_deterministic_binning(leg):
     c = synth.config("c2", n=50000, W=320, H=240)
     sc, cam = c["scene"], c["camera"]
