@@ -8,8 +8,9 @@
 // smooth_kernel: persistent, one CTA per SM, tiles of 128 Gaussians one after
 // another.  Four warpgroups serve the tile's 128 rows (TMEM lanes), each
 // taking 32 of every 128-column epilogue's columns; the loss epilogue is
-// warpgroup 0's.  Warp 0 issues each tcgen05.mma round; after it completes,
-// all threads run its epilogue (bias and ReLU, or the ReLU's mask, BF16 into
+// warpgroup 0's.  A warp of its own issues each tcgen05.mma round (an epilogue
+// warp that does is held up while the MMAs queue); after it completes, the
+// warpgroups run its epilogue (bias and ReLU, or the ReLU's mask, BF16 into
 // shared memory):
 //   forward  H1 = relu(X W1^T + b1), H2, H3, Z = H3 W4^T + b4 (FP32 accumulation)
 //   loss     per row: diff = Z - s_G, n = |diff|; dZ = lambda/n_total diff/n;
@@ -17,7 +18,8 @@
 //   backward dH3 = (dZ W4) o [H3 > 0], dH2 = (dH3 W3) o [H2 > 0], dH1 = ...,
 //            in a buffer of their own and in H3's, so that a round's weight
 //            gradients, which read the layer outputs, run under the epilogue of
-//            its input gradient (1M Gaussians 0.490 -> 0.467 ms).  Weight gradients
+//            its input gradient (1M Gaussians 0.490 -> 0.467 ms; with
+//            the MMA warp 0.427).  Weight gradients
 //            dW = dH^T H_prev accumulate in
 //            TMEM over all of a CTA's tiles (MMAs reading both operands
 //            MN-major from the row-major activation buffers, no transposed
@@ -37,7 +39,8 @@ using namespace tc;
 
 constexpr int kH = 128, kS = 8;
 constexpr int kParts = 4;                    // warpgroups per CTA
-constexpr int kThreadsS = 128 * kParts;
+constexpr int kEpiWarps = 4 * kParts;
+constexpr int kThreadsS = 32 * (kEpiWarps + 1);   // and the MMA warp
 // TMEM columns
 constexpr uint32_t kAcc = 0, kDW2 = 128, kDW3 = 256, kDW1 = 384, kDW4 = 400, kDB2 = 416, kDB3 = 432;
 
@@ -67,38 +70,34 @@ constexpr uint32_t kODZ = kOD + sbuf_bytes(128, 128);        // [128][16]
 constexpr uint32_t kOE = kODZ + sbuf_bytes(128, 16);         // [128][16], column 0 = 1
 constexpr uint32_t kOB = kOE + sbuf_bytes(128, 16);          // biases FP32: b1, b2, b3 (128 each), b4 (8)
 constexpr uint32_t kOBar = kOB + (3 * kH + 16) * 4;
-constexpr uint32_t kSmoothSmem = kOBar + 32 + 1024;
+constexpr uint32_t kSmoothSmem = kOBar + 48 + 1024;
 static_assert(kSmoothSmem <= 227 * 1024, "smoothing shared memory");
 
 struct Ctx {
     unsigned char* sm;
     uint32_t s0;                   // shared address of sm
-    uint64_t* bar;
+    // a round's operands written, one arrival per epilogue warp (even and odd rounds, so that a warp that runs
+    // ahead from the last round of a tile into the next tile's first one does not count for another); its result
+    uint64_t *ready, *done;
     uint32_t* tslot;
     uint32_t phase;
     uint32_t tmem, lanef;
     int row;
-    bool issuer;                   // warp 0 (warp-uniform)
     int part;                      // warpgroup: columns [32 part, 32 part + 32) of each hidden epilogue
 };
 
-// Wait for the MMA round just committed; every thread agrees on the outcome.
-__device__ __forceinline__ bool round_wait(Ctx& c)
-{
-    const bool ok = mbar_wait(c.bar, c.phase);
-    c.phase ^= 1u;
-    const bool bad = __syncthreads_or(!ok);
-    fence_after();
-    return !bad;
-}
-
-// Shared-memory writes visible to the tensor core, TMEM reads ordered before the next MMAs.
-__device__ __forceinline__ void publish()
+// This warp's shared-memory writes are visible to the tensor core and its TMEM
+// reads ordered before the next MMAs; then wait for those.
+__device__ __forceinline__ bool next_round(Ctx& c, int round)
 {
     fence_proxy_async();
     fence_before();
-    __syncthreads();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(c.ready + (round & 1));
+    const bool ok = warp_agree(mbar_wait(c.done, c.phase));
+    c.phase ^= 1u;
     fence_after();
+    return ok;
 }
 
 // This warpgroup's 32 columns of the epilogue of a 128-column hidden layer:
@@ -136,40 +135,40 @@ __device__ __forceinline__ uint64_t kd(uint32_t s0, uint32_t off, int C) { retur
 // MN-major descriptor (rows = K) of a C-column buffer.
 __device__ __forceinline__ uint64_t md(uint32_t s0, uint32_t off, int C) { return mndesc_at(s0 + off, C, 0, 0); }
 
-// One MMA round, issued by warp 0's elected lane.  K steps of 16 move the start
-// address by 16 units (K-major) or 2C units (MN-major over a C-column buffer).
-// The commit follows the MMAs whose result the next epilogue reads; the weight
-// gradients behind it run under that epilogue (they are complete by the next
-// round's commit, which is before anything they read is written again) and the
-// last round, dW1, under the next tile's first one.  x: this tile's X.
+// One MMA round, issued by the MMA warp's elected lane.  K steps of 16 move the
+// start address by 16 units (K-major) or 2C units (MN-major over a C-column
+// buffer).  The commit follows the MMAs whose result the next epilogue reads;
+// the weight gradients behind it run under that epilogue (they are complete by
+// the next round's commit, which is before anything they read is written again)
+// and the last round, dW1, under the next tile's first one.  x: this tile's X.
 __device__ __forceinline__ void issue(const Ctx& c, int round, bool first_tile, uint32_t x)
 {
-    if (!c.issuer || !elect_one()) return;
+    if (!elect_one()) return;
     const uint32_t s0 = c.s0, t = c.tmem;
     const uint32_t keep = first_tile ? 0u : 1u;
     switch (round) {
         case 0:   // H1 pre-activation = X W1^T
             mma(t + kAcc, kd(s0, x, 16), kd(s0, kOW1, 16), idesc_bf16(kH, false, false), 0u);
-            commit(c.bar);
+            commit(c.done);
             break;
         case 1:   // H2 = H1 W2^T
         case 2: { // H3 = H2 W3^T
             const uint64_t a = kd(s0, round == 1 ? kOH1 : kOH2, kH), b = kd(s0, round == 1 ? kOW2 : kOW3, kH);
 #pragma unroll
             for (int k = 0; k < 8; ++k) mma(t + kAcc, a + 16 * k, b + 16 * k, idesc_bf16(kH, false, false), k > 0);
-            commit(c.bar);
+            commit(c.done);
             break;
         }
         case 3: { // Z = H3 W4^T (N = 16, 8 used)
             const uint64_t a = kd(s0, kOH3, kH), b = kd(s0, kOW4, kH);
 #pragma unroll
             for (int k = 0; k < 8; ++k) mma(t + kAcc, a + 16 * k, b + 16 * k, idesc_bf16(16, false, false), k > 0);
-            commit(c.bar);
+            commit(c.done);
             break;
         }
         case 4: { // dH3 (pre-mask) = dZ W4; dW4^T += H3^T dZ
             mma(t + kAcc, kd(s0, kODZ, 16), md(s0, kOW4, kH), idesc_bf16(kH, false, true), 0u);
-            commit(c.bar);
+            commit(c.done);
             const uint64_t a = md(s0, kOH3, kH), b = md(s0, kODZ, 16);
 #pragma unroll
             for (int k = 0; k < 8; ++k)
@@ -183,7 +182,7 @@ __device__ __forceinline__ void issue(const Ctx& c, int round, bool first_tile, 
             const uint64_t ak = kd(s0, dh, kH), wm = md(s0, w, kH);
 #pragma unroll
             for (int k = 0; k < 8; ++k) mma(t + kAcc, ak + 16 * k, wm + 256 * k, idesc_bf16(kH, false, true), k > 0);
-            commit(c.bar);
+            commit(c.done);
             const uint64_t am = md(s0, dh, kH), hm = md(s0, hp, kH), em = md(s0, kOE, 16);
 #pragma unroll
             for (int k = 0; k < 8; ++k)
@@ -231,13 +230,14 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
     Ctx c;
     c.sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     c.s0 = smem_u32(c.sm);
-    c.bar = reinterpret_cast<uint64_t*>(c.sm + kOBar);
-    c.tslot = reinterpret_cast<uint32_t*>(c.sm + kOBar + 16);
+    c.ready = reinterpret_cast<uint64_t*>(c.sm + kOBar);
+    c.done = c.ready + 2;
+    uint64_t* const fin = c.ready + 3;
+    c.tslot = reinterpret_cast<uint32_t*>(c.sm + kOBar + 32);
     c.phase = 0;
     c.row = threadIdx.x & 127;
     c.part = threadIdx.x >> 7;
     const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    c.issuer = warp == 0;
     c.lanef = (uint32_t)(32 * (warp & 3)) << 16;
     // weights (BF16, [out][in]), biases (FP32), the ones operand
     sbuf_fill(SBuf{c.sm + kOW1, 16}, 128, a.W1, 3, kH, 3);
@@ -253,7 +253,12 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
         sbuf_store8(SBuf{c.sm + kOE, 16}, c.row, 0, v);
         sbuf_store8(SBuf{c.sm + kOE, 16}, c.row, 8, z);
     }
-    if (threadIdx.x == 0) mbar_init(c.bar, 1);
+    if (threadIdx.x == 0) {
+        mbar_init(c.ready, kEpiWarps);
+        mbar_init(c.ready + 1, kEpiWarps);
+        mbar_init(c.done, 1);
+        mbar_init(fin, 1);
+    }
     if (warp == 0) tmem_alloc(c.tslot, 512);
     fence_proxy_async();
     fence_before();
@@ -265,10 +270,29 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
     const float* b2 = bs + kH;
     const float* b3 = bs + 2 * kH;
     const float* b4 = bs + 3 * kH;
-    float lsum = 0.f, db4acc = 0.f;
+    double lsum = 0.0;                           // one add per row and tile
+    float db4acc = 0.f;
     bool ok = true, any = false, odd = false;
-    for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
-        const bool first = !any;
+    if (warp == kEpiWarps) {
+        // every round's operands are ready once the epilogue warps have signalled
+        for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+            const uint32_t x = kOX + (odd ? sbuf_bytes(128, 16) : 0u);
+#pragma unroll
+            for (int round = 0; round < 8 && ok; ++round) {
+                ok = warp_agree(mbar_wait(c.ready + (round & 1), (uint32_t)(round >> 1) & 1u));
+                fence_after();
+                if (ok) issue(c, round, !any, x);
+                __syncwarp();
+            }
+            any = true;
+            odd = !odd;
+        }
+        // nothing of ours may still be running when TMEM is read for the flush, or freed
+        if (elect_one()) commit(fin);
+        ok = mbar_wait(fin, 0) && ok;
+        any = false;                             // no rows to flush
+    }
+    for (int t = blockIdx.x; warp < kEpiWarps && t < a.ntiles && ok; t += gridDim.x) {
         any = true;
         const uint32_t x = kOX + (odd ? sbuf_bytes(128, 16) : 0u);
         odd = !odd;
@@ -299,21 +323,13 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
             sbuf_store8(SBuf{c.sm + x, 16}, c.row, 0, v);
             sbuf_store8(SBuf{c.sm + x, 16}, c.row, 8, z);
         }
-        publish();
-        issue(c, 0, first, x);
-        if (!(ok = round_wait(c))) break;
+        if (!(ok = next_round(c, 0))) break;
         hidden_epilogue(c, b1, kOH1);
-        publish();
-        issue(c, 1, first, x);
-        if (!(ok = round_wait(c))) break;
+        if (!(ok = next_round(c, 1))) break;
         hidden_epilogue(c, b2, kOH2);
-        publish();
-        issue(c, 2, first, x);
-        if (!(ok = round_wait(c))) break;
+        if (!(ok = next_round(c, 2))) break;
         hidden_epilogue(c, b3, kOH3);
-        publish();
-        issue(c, 3, first, x);
-        if (!(ok = round_wait(c))) break;
+        if (!(ok = next_round(c, 3))) break;
         if (p0) {   // loss and the output gradient
             float z[16];
             tmem_ld16(c.tmem + c.lanef + kAcc, z);
@@ -327,7 +343,7 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
             }
             nn = sqrtf(nn);
             const float wgt = valid ? fmaxf(ug, a.w_s) : 0.f;
-            lsum += (1.f + wgt) * nn;
+            lsum += (double)((1.f + wgt) * nn);
             const float inv = nn > 0.f ? a.scale / nn : 0.f;
             float dz[16];
 #pragma unroll
@@ -339,36 +355,24 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
             sbuf_store8(SBuf{c.sm + kODZ, 16}, c.row, 8, dz + 8);
             db4acc += colsum16(dz, lane);       // lanes 2k, 2k+1: column k (k < 8)
         }
-        publish();
-        issue(c, 4, first, x);
-        if (!(ok = round_wait(c))) break;
+        if (!(ok = next_round(c, 4))) break;
         grad_epilogue(c, kOH3, kOD);         // dH3
-        publish();
-        issue(c, 5, first, x);
-        if (!(ok = round_wait(c))) break;
+        if (!(ok = next_round(c, 5))) break;
         grad_epilogue(c, kOH2, kOH3);        // dH2 over H3 (read by dW4, complete)
-        publish();
-        issue(c, 6, first, x);
-        if (!(ok = round_wait(c))) break;
+        if (!(ok = next_round(c, 6))) break;
         grad_epilogue(c, kOH1, kOD);         // dH1 over dH3 (read by dW3, complete)
-        publish();
-        issue(c, 7, first, x);
+        // dW1: nothing here waits for it
+        fence_proxy_async();
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(c.ready + 1);
     }
-    if (ok && any) {                             // the last tile's dW1
-        if (c.issuer && elect_one()) commit(c.bar);
-        ok = round_wait(c);
-    }
+    if (warp < kEpiWarps) ok = warp_agree(mbar_wait(fin, 0)) && ok;
+    fence_after();
+    ok = !__syncthreads_or(!ok);
     if (!ok) {
-        if (c.issuer) {
-            // nothing of ours may still be running when TMEM is freed
-            if (elect_one()) {
-                atomicExch(&g_smooth_error, 1);
-                commit(c.bar);
-            }
-            (void)mbar_wait(c.bar, c.phase);
-        }
+        if (threadIdx.x == 0) atomicExch(&g_smooth_error, 1);
     } else if (any) {
-        // flush: TMEM lane = this thread's row of each accumulator
         // flush: TMEM lane = this thread's row of each accumulator; warpgroup p takes
         // columns [32 p, 32 p + 32) of dW2 and dW3 and one of the small blocks
         float v[16];
@@ -401,7 +405,12 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
         if (c.part == 0) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-            if (lane == 0) atomicAdd(a.loss, lsum * a.scale);
+            // one FP32 add per CTA: the order of several hundred showed in the loss at 1e-6
+            double* const part = reinterpret_cast<double*>(c.sm + kODZ);
+            if (lane == 0) part[warp] = lsum;
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (threadIdx.x == 0)
+                atomicAdd(a.loss, (float)((part[0] + part[1] + part[2] + part[3]) * (double)a.scale));
             if ((lane & 1) == 0 && (lane >> 1) < kS) atomicAdd(a.db4 + (lane >> 1), db4acc);
         }
     }
