@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
 //   S6  dx  = dh1 W1; [dW1 | db1] += dh1^T [x | 1]     E6  dx -> d_feat
 // dz, dh2 and dh1 are stored pixel-major: the input-gradient MMAs read them
 // K-major and the weight-gradient MMAs MN-major (contracting over the tile's
-// pixels).  Handshake per slot: its 256 epilogue threads arrive on ready[s]
+// pixels).  Handshake per slot: its eight epilogue warps arrive on ready[s]
 // once their operand is in shared memory and their TMEM reads are done; the
 // MMA thread waits, issues, and commits to done[s].  All MMAs come from one
 // thread, so the weight-gradient accumulations of both slots are ordered.
@@ -459,7 +459,8 @@ __device__ __forceinline__ void epi_signal(const EpiCtx& e)
 {
     fence_proxy_async();
     fence_before();
-    mbar_arrive(e.ready);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(e.ready);
 }
 
 // Wait for the slot's MMAs; the outcome is made uniform over the slot's 256
@@ -715,8 +716,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) dec_train_kernel(DecArgs a)
         sbuf_store8(E, r, 8 * cb, v);
     }
     if (threadIdx.x == 0) {
-        mbar_init(ready, 256);
-        mbar_init(ready + 1, 256);
+        mbar_init(ready, 8);
+        mbar_init(ready + 1, 8);
         mbar_init(done, 1);
         mbar_init(done + 1, 1);
         mbar_init(fin, 1);
