@@ -99,7 +99,7 @@ struct Smem {
     uint64_t *full, *empty, *acc_full, *acc_empty, *norm_ready, *norm_free, *fin;
     float* norms;                // [2 slots][2][128] inverse feature norms
     float* xch;                  // [2 slots][parts][4][128] epilogue exchange
-    float* rv;                   // [N] utilisation ratio (gradient mode)
+    float* rv;                   // [N] utilisation ratio (gradient mode); else four FP64 sums
     float* inv_s;                // [2][N]
     unsigned* cnt;               // [N]
     uint32_t* tmem_slot;
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(threads_of(GRAD), 1) quant_kernel(const __grid
         float psum[kPC], usum[kPC];   // softmax column sums (gradient mode: sums of g cos^C, g cos^D)
 #pragma unroll
         for (int i = 0; i < kPC; ++i) psum[i] = usum[i] = 0.f;
-        float lcos = 0.f;
+        double lcos = 0.0;                        // one add per row
         int it = 0;
         for (int t = blockIdx.x; t < q.ntiles && ok; t += gridDim.x, ++it) {
             const int slot = it & 1;
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(threads_of(GRAD), 1) quant_kernel(const __grid
                 mbar_arrive(s.acc_empty + slot);
                 if (valid && h == 0) {
                     q.m_out[row] = bi;
-                    lcos += 1.0f + q.lambda_d - best;
+                    lcos += (double)(1.0f + q.lambda_d - best);
                     atomicAdd(s.cnt + bi, 1u);
                 }
             }
@@ -585,7 +585,8 @@ __global__ void __launch_bounds__(threads_of(GRAD), 1) quant_kernel(const __grid
                             atomicAdd(q.u + N + 16 * (c_lo + cc) + (lane >> 1), usum[cc]);
                         }
             } else {
-                if (lane == 0 && h == 0) atomicAdd(q.lcos, lcos);
+                // the quadrants' sums, added to the output once per CTA below
+                if (lane == 0 && h == 0) reinterpret_cast<double*>(s.rv)[quad] = lcos;
                 if ((lane & 1) == 0)
 #pragma unroll
                     for (int cc = 0; cc < kPC; ++cc)
@@ -601,6 +602,8 @@ __global__ void __launch_bounds__(threads_of(GRAD), 1) quant_kernel(const __grid
     } else if (!GRAD) {
         for (int i = threadIdx.x; i < N; i += blockDim.x)
             if (s.cnt[i]) atomicAdd(q.count + i, s.cnt[i]);
+        const double* part = reinterpret_cast<const double*>(s.rv);
+        if (threadIdx.x == 0) atomicAdd(q.lcos, (float)((part[0] + part[1]) + (part[2] + part[3])));
     }
     if (warp == 1) tmem_dealloc(tmem, ncols);
 }
