@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kBlock / 2, 8) render_fwd_phase_kernel(
     }
 }
 
-// Four pixels per thread -- rows y, y + 2, y + 4, y + 6 of one column, warp w
+// PPT pixels per thread, U records at a time.  <4, 1>: rows y, y + 2, y + 4, y + 6 of one column, warp w
 // covering the compact 16 x 8 block of rows [8w, 8w + 8) -- in two pairs
 // (y, y + 2) and (y + 4, y + 6) whose arithmetic runs on paired FP32
 // instructions.  The channel contractions pair channels instead: per Gaussian
@@ -272,20 +272,20 @@ __global__ void __launch_bounds__(kBlock / 2, 8) render_fwd_phase_kernel(
 // column's dx, come from three sums over the thread's pixels -- D = sum dP,
 // E = sum dP dy, F = sum dP dy^2 with dP = dL/dpower -- formed once per record:
 // dconic = (-dx^2 D / 2, -dx E, -F / 2), dmean = (-A dx D - B E, -C E - B dx D).
-template <int PPT>
+template <int PPT, int U>
 __global__ void __launch_bounds__(kBlock / PPT) render_bwd_kernel(
     CamParams cam, const float4* __restrict__ splat, const uint32_t* __restrict__ ids, const uint2* __restrict__ ranges,
     const float* __restrict__ T_final, const int* __restrict__ n_contrib, const float* __restrict__ dL_drgb,
     const float* __restrict__ dL_dfeat, const float* __restrict__ dL_dunc, float4* __restrict__ grad2d)
 {
-    static_assert(PPT == 4, "two pixel pairs per thread");
-    constexpr int NT = kBlock / PPT;
+    static_assert(PPT == 2 || PPT == 4, "one or two pixel pairs per thread");
+    constexpr int NT = kBlock / PPT, NPR = PPT / 2;
     __shared__ float4 rec[5][kBlock];
     __shared__ uint32_t sid[kBlock];
     __shared__ int s_max;
     // per warp, the lanes' 18 gradient partial sums, field-major; the row stride
     // of 36 floats staggers the rows over the banks for the 16-byte reads
-    __shared__ __align__(16) float red[NT / 32][18][36];
+    __shared__ __align__(16) float red[NT / 32][18 * U][36];
     const int tile = blockIdx.x;
     const int tx = tile % cam.TX, ty = tile / cam.TX;
     const int px = tx * LE_TILE + (threadIdx.x & 15);
@@ -296,12 +296,12 @@ __global__ void __launch_bounds__(kBlock / PPT) render_bwd_kernel(
 
     // pair p holds pixels q = 2p (x) and 2p + 1 (y); dC[q][k] = pixel q's upstream
     // gradient of channels (2k, 2k + 1)
-    float2 npy[2], dC[PPT][6], T[2], Tf[2], S[2], nbg[2];
+    float2 npy[NPR], dC[PPT][6], T[NPR], Tf[NPR], S[NPR], nbg[NPR];
     int last[PPT];
     int lmax = 0;
 #pragma unroll
     for (int q = 0; q < PPT; ++q) {
-        const int y = ty * LE_TILE + 8 * (threadIdx.x >> 5) + ((threadIdx.x >> 4) & 1) + 2 * q;
+        const int y = ty * LE_TILE + 2 * PPT * (threadIdx.x >> 5) + ((threadIdx.x >> 4) & 1) + 2 * q;
         const bool inside = px < cam.W && y < cam.H;
         const size_t o = (size_t)y * cam.W + px;
         float d[12];
@@ -355,46 +355,64 @@ __global__ void __launch_bounds__(kBlock / PPT) render_bwd_kernel(
             }
         }
         __syncthreads();
-        for (int j = min(b_end, wmax) - b_start - 1; j >= 0; --j) {
-            const int pos = b_start + j;
-            const float4 g0 = rec[0][j], g1 = rec[1][j];
-            const float dx = __fsub_rn(g0.x, fpx);
-            const float ax = splat_ax(g0.z, dx), bx = splat_bx(g0.w, dx);
-            // the forward kernel's skip decisions, per pixel, with identical roundings
-            float2 dy[2], G[2], al[2], a0[2];
-            bool cb[PPT], any_mine = false;
+        for (int j0 = min(b_end, wmax) - b_start - 1; j0 >= 0; j0 -= U) {
+            // the forward kernel's skip decisions for U records, per pixel, with identical roundings
+            float4 g0[U], g1[U];
+            float dx[U];
+            float2 dy[U][NPR], G[U][NPR], al[U][NPR], a0[U][NPR];
+            bool cb[U][PPT], any_mine[U], warp_any[U];
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                dy[p] = __fadd2_rn(f2(g0.y), npy[p]);
-                const float2 qq = __ffma2_rn(f2(g1.x), __fmul2_rn(dy[p], dy[p]), __ffma2_rn(f2(bx), dy[p], f2(ax)));
-                G[p] = make_float2(ex2_approx(-qq.x), ex2_approx(-qq.y));
-                a0[p] = __fmul2_rn(f2(g1.y), G[p]);
-                al[p] = make_float2(fminf(0.99f, a0[p].x), fminf(0.99f, a0[p].y));
-                cb[2 * p] = pos < last[2 * p] && qq.x >= 0.f && al[p].x >= (1.f / 255.f);
-                cb[2 * p + 1] = pos < last[2 * p + 1] && qq.y >= 0.f && al[p].y >= (1.f / 255.f);
-                any_mine = any_mine || cb[2 * p] || cb[2 * p + 1];
+            for (int u = 0; u < U; ++u) {
+                const int j = U == 1 ? j0 : max(j0 - u, 0);
+                const int pos = b_start + j0 - u;
+                g0[u] = rec[0][j];
+                g1[u] = rec[1][j];
+                dx[u] = __fsub_rn(g0[u].x, fpx);
+                const float ax = splat_ax(g0[u].z, dx[u]), bx = splat_bx(g0[u].w, dx[u]);
+                any_mine[u] = false;
+#pragma unroll
+                for (int p = 0; p < NPR; ++p) {
+                    dy[u][p] = __fadd2_rn(f2(g0[u].y), npy[p]);
+                    const float2 qq = __ffma2_rn(f2(g1[u].x), __fmul2_rn(dy[u][p], dy[u][p]),
+                                                 __ffma2_rn(f2(bx), dy[u][p], f2(ax)));
+                    G[u][p] = make_float2(ex2_approx(-qq.x), ex2_approx(-qq.y));
+                    a0[u][p] = __fmul2_rn(f2(g1[u].y), G[u][p]);
+                    al[u][p] = make_float2(fminf(0.99f, a0[u][p].x), fminf(0.99f, a0[u][p].y));
+                    const bool here = U == 1 || j0 - u >= 0;
+                    cb[u][2 * p] = here && pos < last[2 * p] && qq.x >= 0.f && al[u][p].x >= (1.f / 255.f);
+                    cb[u][2 * p + 1] = here && pos < last[2 * p + 1] && qq.y >= 0.f && al[u][p].y >= (1.f / 255.f);
+                    any_mine[u] = any_mine[u] || cb[u][2 * p] || cb[u][2 * p + 1];
+                }
+                warp_any[u] = __any_sync(0xffffffffu, any_mine[u]);
             }
-            if (!__any_sync(0xffffffffu, any_mine)) continue;
-            float gr[18];
-            {
+            bool some = warp_any[0];
+#pragma unroll
+            for (int u = 1; u < U; ++u) some = some || warp_any[u];
+            if (!some) continue;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int j = U == 1 ? j0 : max(j0 - u, 0);
+                float gr[18];
                 // acc[k]: channels (2k, 2k + 1) of sum_q w_q dL/dC_q over the thread's pixels
                 float2 acc[6], sD = f2(0.f), sE = f2(0.f), sF = f2(0.f), sO = f2(0.f);
 #pragma unroll
                 for (int k = 0; k < 6; ++k) acc[k] = f2(0.f);
-                if (any_mine) {
+                // several records go through without a branch, so that their chains overlap; a thread none of
+                // whose pixels blends one contributes zeros to it
+                if (U > 1 || any_mine[u]) {
                     const float4 g2 = rec[2][j], g3 = rec[3][j], g4 = rec[4][j];
                     // the record's channels in the pairs its 16-byte words already hold
-                    const float2 fp[6] = {make_float2(g1.z, g1.w), make_float2(g2.x, g2.y),
+                    const float2 fp[6] = {make_float2(g1[u].z, g1[u].w), make_float2(g2.x, g2.y),
                                           make_float2(g2.z, g2.w), make_float2(g3.x, g3.y),
                                           make_float2(g3.z, g3.w), make_float2(g4.x, g4.y)};
 #pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        const bool cx = cb[2 * p], cy = cb[2 * p + 1];
+                    for (int p = 0; p < NPR; ++p) {
+                        const bool cx = cb[u][2 * p], cy = cb[u][2 * p + 1];
                         // alpha of the blended pixels, 0 for the others (1 / (1 - 0) = 1 leaves T,
-                        // and w, dP and the opacity term are 0): both pairs run straight-line, which
-                        // keeps the kernel at 127 registers (8 blocks per SM; a branch per pair took
+                        // and w, dP and the opacity term are 0): the pairs run straight-line, which
+                        // keeps the four-pixel kernel at 127 registers (8 blocks per SM; a branch per pair took
                         // 168 registers, 6 blocks, and 11 % more time at 1M Gaussians)
-                        const float2 am = sel2(cx, cy, al[p]);
+                        const float2 am = sel2(cx, cy, al[u][p]);
                         const float2 inv = make_float2(__fdividef(1.f, 1.f - am.x), __fdividef(1.f, 1.f - am.y));
                         T[p] = __fmul2_rn(T[p], inv);
                         const float2 w = __fmul2_rn(am, T[p]);
@@ -416,23 +434,23 @@ __global__ void __launch_bounds__(kBlock / PPT) render_bwd_kernel(
                         const float2 dal = __ffma2_rn(T[p], diff, __fmul2_rn(__fmul2_rn(Tf[p], inv), nbg[p]));
                         S[p] = __ffma2_rn(am, diff, S[p]);
                         // alpha below the 0.99 clamp: dalpha/dpower = alpha, dalpha/do = G
-                        const bool mx = cx && a0[p].x < 0.99f, my = cy && a0[p].y < 0.99f;
-                        const float2 dP = __fmul2_rn(dal, sel2(mx, my, al[p]));
-                        sO = __ffma2_rn(dal, sel2(mx, my, G[p]), sO);
+                        const bool mx = cx && a0[u][p].x < 0.99f, my = cy && a0[u][p].y < 0.99f;
+                        const float2 dP = __fmul2_rn(dal, sel2(mx, my, al[u][p]));
+                        sO = __ffma2_rn(dal, sel2(mx, my, G[u][p]), sO);
                         sD = __fadd2_rn(sD, dP);
-                        const float2 t = __fmul2_rn(dP, dy[p]);
+                        const float2 t = __fmul2_rn(dP, dy[u][p]);
                         sE = __fadd2_rn(sE, t);
-                        sF = __ffma2_rn(t, dy[p], sF);
+                        sF = __ffma2_rn(t, dy[u][p], sF);
                     }
                 }
                 // the conic itself, for the mean gradient (dL/dpower is per unit of the natural exponent)
-                const float cA = g0.z * kConicUnscaleAC, cB = g0.w * kConicUnscaleB, cC = g1.x * kConicUnscaleAC;
+                const float cA = g0[u].z * kConicUnscaleAC, cB = g0[u].w * kConicUnscaleB, cC = g1[u].x * kConicUnscaleAC;
                 const float D = sD.x + sD.y, E = sE.x + sE.y, F = sF.x + sF.y;
-                const float dxD = dx * D;
+                const float dxD = dx[u] * D;
                 gr[0] = -(cA * dxD + cB * E);
                 gr[1] = -(cC * E + cB * dxD);
-                gr[2] = -0.5f * dx * dxD;
-                gr[3] = -dx * E;
+                gr[2] = -0.5f * dx[u] * dxD;
+                gr[3] = -dx[u] * E;
                 gr[4] = -0.5f * F;
                 gr[5] = sO.x + sO.y;
 #pragma unroll
@@ -440,22 +458,27 @@ __global__ void __launch_bounds__(kBlock / PPT) render_bwd_kernel(
                     gr[6 + 2 * k] = acc[k].x;
                     gr[7 + 2 * k] = acc[k].y;
                 }
-            }
-            // warp sums of the 18 fields: a transpose through shared memory, lane f < 18 adding field f
+                // warp sums of the 18 fields: a transpose through shared memory, lane f < 18 adding field f
 #pragma unroll
-            for (int c = 0; c < 18; ++c) wred[c][lane] = gr[c];
+                for (int c = 0; c < 18; ++c) wred[18 * u + c][lane] = U == 1 || any_mine[u] ? gr[c] : 0.f;
+            }
             __syncwarp();
             if (lane < 18) {
-                const float4* row = reinterpret_cast<const float4*>(wred[lane]);
-                float2 a = f2(0.f), b = f2(0.f);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float4 v = row[k];
-                    a = __fadd2_rn(a, make_float2(v.x, v.y));
-                    b = __fadd2_rn(b, make_float2(v.z, v.w));
+                for (int u = 0; u < U; ++u) {
+                    if (U > 1 && !warp_any[u]) continue;
+                    const float4* row = reinterpret_cast<const float4*>(wred[18 * u + lane]);
+                    float2 a = f2(0.f), b = f2(0.f);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float4 v = row[k];
+                        a = __fadd2_rn(a, make_float2(v.x, v.y));
+                        b = __fadd2_rn(b, make_float2(v.z, v.w));
+                    }
+                    const float2 t = __fadd2_rn(a, b);
+                    atomicAdd(reinterpret_cast<float*>(grad2d + (size_t)sid[U == 1 ? j0 : max(j0 - u, 0)] * 5) + lane,
+                              t.x + t.y);
                 }
-                const float2 t = __fadd2_rn(a, b);
-                atomicAdd(reinterpret_cast<float*>(grad2d + (size_t)sid[j] * 5) + lane, t.x + t.y);
             }
             __syncwarp();
         }
@@ -504,6 +527,12 @@ extern "C" le_status le_render_fwd(const le_camera* cam, int32_t n, const float*
 namespace leg {
 namespace {
 
+// Up to four tiles per SM, a tile's serial walk sets the time: two pixels per
+// thread, two records at a time.  Backward of 64 / 260 / 600 tiles: 68 / 94 / 121
+// us, with four pixels and one record 99 / 107 / 134; at 1,200 tiles it depends on
+// the scene (191 against 213, 206 against 173), and at 4,293 it is 472 against 393.
+constexpr int kFewTiles = 608;
+
 // Arguments shared by le_render_bwd and le_render_bwd_adam; launches the
 // screen-space backward (grad2d).
 le_status render_backward_2d(const le_camera* cam, const le_gaussians* g, const le_projected* pr,
@@ -513,10 +542,13 @@ le_status render_backward_2d(const le_camera* cam, const le_gaussians* g, const 
 {
     const CamParams cp = cam_params(cam);
     LE_CUDA(cudaMemsetAsync(grad2d, 0, sizeof(float) * LE_SPLAT_STRIDE * (size_t)g->n, s));
-    render_bwd_kernel<4><<<cp.TX * cp.TY, kBlock / 4, 0, s>>>(cp, reinterpret_cast<const float4*>(pr->splat), sorted_ids,
-                                                        reinterpret_cast<const uint2*>(tile_ranges), T_final,
-                                                        n_contrib, dL_drgb, dL_dfeat, dL_dunc,
-                                                        reinterpret_cast<float4*>(grad2d));
+    const auto run = [&](auto kernel, int threads) {
+        kernel<<<cp.TX * cp.TY, threads, 0, s>>>(cp, reinterpret_cast<const float4*>(pr->splat), sorted_ids,
+                                                 reinterpret_cast<const uint2*>(tile_ranges), T_final, n_contrib,
+                                                 dL_drgb, dL_dfeat, dL_dunc, reinterpret_cast<float4*>(grad2d));
+    };
+    if (cp.TX * cp.TY <= kFewTiles) run(render_bwd_kernel<2, 2>, kBlock / 2);
+    else run(render_bwd_kernel<4, 1>, kBlock / 4);
     LE_LAUNCHED();
     return LE_OK;
 }

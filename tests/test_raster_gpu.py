@@ -103,6 +103,26 @@ def test_backward_parity(leg, orc, case):
     assert rel_err(to_np(grads.unc), g2["unc"]) < 1e-4
 
 
+@pytest.mark.parametrize("W,H", [(16, 16), (37, 21), (608, 256), (624, 256)])
+def test_backward_few_and_many_tiles(leg, orc, W, H):
+    """The backward's two layouts on both sides of their line (608 tiles) and on odd list lengths, against
+    the oracle's adjoint: 1e-4 of each field's largest gradient."""
+    c = synth.config("c1", n=601, W=W, H=H)
+    sc, cam = c["scene"], c["camera"]
+    cam.bg = np.array([0.3, 0.1, 0.2], np.float32)
+    ref = orc.forward(sc, cam)
+    ok = ref["img"]["flip"] == 0
+    dr, df, du = upstream(np.random.default_rng(W), H, W, ok)
+    g, proj, ids, ranges, K, keys, img = _run(leg, sc, cam)
+    grads, _ = leg.le_render_bwd(cam, g, proj, ids, ranges, img, _t(dr), _t(df), _t(du))
+    g2 = orc.render_bwd(cam, sc, ref["proj"], ref["vals"], ref["ranges"], dr, df, du)
+    gp = orc.project_bwd(sc, cam, ref["kp"]["tiles"], g2["mean2d"], g2["conic"], g2["opacity"], g2["rgb"])
+    for k in ("means", "log_scales", "quats", "opacity_raw", "sh"):
+        assert rel_err(to_np(getattr(grads, k)), gp[k]) < 1e-4, k
+    assert rel_err(to_np(grads.feat), g2["feat"]) < 1e-4
+    assert rel_err(to_np(grads.unc), g2["unc"]) < 1e-4
+
+
 def test_autograd_function(leg, orc):
     c = synth.config("c1", n=800, W=64, H=64)
     sc, cam = c["scene"], c["camera"]
