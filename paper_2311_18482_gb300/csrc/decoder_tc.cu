@@ -765,13 +765,10 @@ __global__ void __launch_bounds__(kTrainThreads, 1) dec_train_kernel(DecArgs a)
         for (int k = 0; k < 2; ++k) {
             tmem_ld16(tb + kTW3 + lanef + 32 * wg + 16 * k, v);
             if (row < a.ncb)
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    atomicAdd(a.dW3 + (size_t)row * kH2 + 32 * wg + 16 * k + j, v[j] * a.invP);
+                red_row<16>(a.dW3 + (size_t)row * kH2 + 32 * wg + 16 * k, v, a.invP, red_vec(a.dW3));
         }
         tmem_ld16(tb + kTW2 + lanef + 16 * wg, v);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) atomicAdd(a.dW2 + (size_t)row * kH1 + 16 * wg + j, v[j] * a.invP);
+        red_row<16>(a.dW2 + (size_t)row * kH1 + 16 * wg, v, a.invP, red_vec(a.dW2));
         if (wg == 0) {
             tmem_ld16(tb + kTP + lanef, v);
             atomicAdd(a.db2 + row, v[0] * a.invP);
@@ -779,8 +776,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) dec_train_kernel(DecArgs a)
         } else if (wg == 1) {
             tmem_ld16(tb + kTQ + lanef, v);
             if (row < kH1) {
-#pragma unroll
-                for (int j = 0; j < kD; ++j) atomicAdd(a.dW1 + (size_t)row * kD + j, v[j] * a.invP);
+                red_row<kD>(a.dW1 + (size_t)row * kD, v, a.invP, red_vec(a.dW1));
                 atomicAdd(a.db1 + row, v[kD] * a.invP);
             }
         }
@@ -1415,7 +1411,7 @@ extern "C" le_status le_feature_map_workspace(int32_t n_cb, int32_t d, size_t* b
     LE_TRACE("le_feature_map_workspace");
     LE_CHECK_ARG(bytes != nullptr, "bytes is null");
     LE_CHECK_ARG(n_cb > 0 && d > 0, "bad sizes");
-    *bytes = (size_t)n_cb * d * 2 + (size_t)n_cb * 128 * 2;   // codebook image + W3 image
+    *bytes = (size_t)n_cb * d * 2 + (size_t)n_cb * 128 * 2;   // the codebook's image; 256 bytes per code to spare
     return LE_OK;
 }
 

@@ -592,9 +592,7 @@ __global__ void __launch_bounds__(kRows, 1) wide_wgrad_kernel(WgradArgs a)
 #pragma unroll 1
             for (int c = 0; c < kW2; c += 16) {
                 tmem_ld16(tl + c, v);
-                if (tid < a.ncb)
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) atomicAdd(a.dW3 + (size_t)tid * kW2 + c + j, v[j] * a.invP);
+                if (tid < a.ncb) red_row<16>(a.dW3 + (size_t)tid * kW2 + c, v, a.invP, red_vec(a.dW3));
             }
             tmem_ld16(tl + 256, v);
             if (tid < a.ncb) atomicAdd(a.db3 + tid, v[0] * a.invP);
@@ -605,16 +603,14 @@ __global__ void __launch_bounds__(kRows, 1) wide_wgrad_kernel(WgradArgs a)
 #pragma unroll 1
                 for (int c = 0; c < kW1; c += 16) {
                     tmem_ld16(tl + 128 * h + c, v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) atomicAdd(a.dW2 + (size_t)r * kW1 + c + j, v[j] * a.invP);
+                    red_row<16>(a.dW2 + (size_t)r * kW1 + c, v, a.invP, red_vec(a.dW2));
                 }
                 tmem_ld16(tl + 256 + 16 * h, v);
                 atomicAdd(a.db2 + r, v[0] * a.invP);
             }
         } else {
             tmem_ld16(tl, v);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) atomicAdd(a.dW1 + (size_t)tid * 8 + c, v[c] * a.invP);
+            red_row<8>(a.dW1 + (size_t)tid * 8, v, a.invP, red_vec(a.dW1));
             atomicAdd(a.db1 + tid, v[8] * a.invP);
         }
     }

@@ -740,8 +740,7 @@ __global__ void __launch_bounds__(kGThreads, 1) quant_grad_gemm_kernel(const __g
                 float v[16];
                 tmem_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + c0c, v);
                 if (j < g.N)
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) atomicAdd(g.raw + (size_t)j * g.d + 128 * dt + c0c + k, v[k]);
+                    red_row<16>(g.raw + (size_t)j * g.d + 128 * dt + c0c, v, 1.f, red_vec(g.raw));
             }
         }
         ok = ok && got;

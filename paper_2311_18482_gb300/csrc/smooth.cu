@@ -380,11 +380,9 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
 #pragma unroll
         for (int q = 2 * c.part; q < 2 * c.part + 2; ++q) {
             tmem_ld16(c.tmem + c.lanef + kDW2 + 16 * q, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) atomicAdd(a.dW2 + (size_t)r * kH + 16 * q + j, v[j]);
+            red_row<16>(a.dW2 + (size_t)r * kH + 16 * q, v, 1.f, red_vec(a.dW2));
             tmem_ld16(c.tmem + c.lanef + kDW3 + 16 * q, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) atomicAdd(a.dW3 + (size_t)r * kH + 16 * q + j, v[j]);
+            red_row<16>(a.dW3 + (size_t)r * kH + 16 * q, v, 1.f, red_vec(a.dW3));
         }
         if (c.part == 0) {
             tmem_ld16(c.tmem + c.lanef + kDW1, v);

@@ -367,6 +367,29 @@ __device__ __forceinline__ void sts_row16(uint32_t addr, const uint32_t* w)
     sts128(addr + 128, w + 4);
 }
 
+// Whether red_row may use 16-byte reductions at p (and at every row of whole 16 bytes behind it).
+__device__ __forceinline__ bool red_vec(const float* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// Adds N sums (times scale) to p[0 .. N): a CTA's accumulator rows into the call's
+// gradient, every CTA into the same addresses.  Lanes hold different rows, so a
+// scalar add is one L2 operation for 4 bytes and 152 CTAs' worth of them took
+// ~35 us at the end of a kernel; 16-byte reductions take a quarter of the operations
+// (decoder training of 307,200 / 1,088,640 pixels 137 / 307 -> 101 / 271 us,
+// smoothing of 1M Gaussians 442 -> 401 us).
+template <int N>
+__device__ __forceinline__ void red_row(float* p, const float* v, float scale, bool vec)
+{
+    if (vec) {
+#pragma unroll
+        for (int j = 0; j < N; j += 4)
+            atomicAdd(reinterpret_cast<float4*>(p + j),
+                      make_float4(v[j] * scale, v[j + 1] * scale, v[j + 2] * scale, v[j + 3] * scale));
+    } else {
+#pragma unroll
+        for (int j = 0; j < N; ++j) atomicAdd(p + j, v[j] * scale);
+    }
+}
+
 // v where the layer output h (16 columns at addr) is positive, else 0, as BF16 pairs.
 __device__ __forceinline__ void relu_mask16(const float* v, uint32_t addr, uint32_t* w)
 {

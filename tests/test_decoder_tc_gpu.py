@@ -152,6 +152,27 @@ def test_fused_train(leg, orc, P, ncb):
         assert v <= bars[k], ("oracle", k, v)
 
 
+@pytest.mark.parametrize("widths,ncb", [((64, 128), 112), ((128, 256), 128)])
+def test_gradients_at_any_alignment(leg, widths, ncb):
+    """Weight gradients that start off a 16-byte boundary (scalar adds) against aligned ones (16-byte adds):
+    the same at most three CTAs' sums per element, added in some order, so within 3 x 2^-24 of the sum of
+    their magnitudes, which 1e-5 of the tensor's largest element covers up to a cancellation of 50."""
+    P = 300
+    dec = _dec_t(synth.decoder_init(3, ncb, *widths))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    feat = torch.randn((8, P), device="cuda", generator=g)
+    unc = torch.rand(P, device="cuda", generator=g)
+    tgt = torch.randint(0, ncb, (P,), device="cuda", generator=g, dtype=torch.int32)
+    ref = leg.le_decode(leg.FUSED_BF16, feat, dec, unc, tgt)
+    off = [torch.full((t.numel() + 1,), float("nan"), device="cuda")[1:].view(t.shape) for t in dec]
+    loss, d_feat, d_unc = torch.empty(2, device="cuda"), torch.empty_like(feat), torch.empty_like(unc)
+    leg.le_decode_raw(leg.FUSED_BF16, P, feat, unc, leg.decoder_struct(*dec), tgt, 1.0, 1.0, loss, d_feat, d_unc,
+                      leg.decoder_grads_struct(off), None, None, None, ref["workspace"])
+    for o, r in zip(off, ref["dW"]):
+        assert o.data_ptr() % 16 and not r.data_ptr() % 16
+        assert float((o - r).abs().max()) <= 1e-5 * float(r.abs().max())
+
+
 def test_fused_train_matches_unfused(leg):
     """Fused BF16 and unfused FP32 training steps agree (same seeded inputs)."""
     import paper_2311_18482_gb300 as L

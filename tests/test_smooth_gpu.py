@@ -126,3 +126,16 @@ def test_smooth_accumulates_into_strided_records(leg, orc, off, stride):
     got = rec[:, off:off + 8].cpu().numpy().astype(np.float64)
     assert np.abs(got - expect).max() <= 2.5e-7 * np.abs(expect).max()
     assert np.abs(dense["d_feat"]).max() > 1e-5
+
+
+def test_gradients_at_any_alignment(leg):
+    """Weight gradients that start off a 16-byte boundary (scalar adds) against aligned ones (16-byte adds):
+    the same three CTAs' sums per element in some order, within 1e-5 of the tensor's largest element."""
+    mlp, means, feat, unc = _inputs(300, 4)
+    vals = [torch.from_numpy(np.ascontiguousarray(getattr(mlp, k), np.float32)).cuda() for k in KEYS]
+    t = [torch.from_numpy(a).cuda() for a in (means, feat, unc)]
+    ref = leg.le_smooth(*t, vals)[2]
+    off = [torch.full((v.numel() + 1,), float("nan"), device="cuda")[1:].view(v.shape) for v in vals]
+    leg.le_smooth(*t, vals, grads=off)
+    for o, r in zip(off, ref):
+        assert float((o - r).abs().max()) <= 1e-5 * float(r.abs().max())
