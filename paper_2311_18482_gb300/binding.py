@@ -195,7 +195,7 @@ def reset_launch_count():
 
 # ---------------------------------------------------------------------------
 def camera_struct(cam) -> LeCamera:
-    floats = lambda a: (C.c_float * len(a))(*(a.tolist() if hasattr(a, "tolist") else map(float, a)))
+    floats = lambda a: (C.c_float * len(a))(*map(float, a.tolist() if hasattr(a, "tolist") else a))
     return LeCamera(floats(cam.view), floats(cam.campos), float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy),
                     int(cam.W), int(cam.H), float(cam.near), floats(cam.bg))
 
