@@ -1231,18 +1231,6 @@ __global__ void selftest_wait_kernel()
     if (threadIdx.x == 0 && !mbar_wait(&bar, 0u)) atomicExch(&g_tc_error, 1);
 }
 
-// Up to eight FP32 arrays set to zero in one launch (block i clears array i).
-struct ZeroList {
-    float* p[8];
-    int n[8];
-};
-__global__ void __launch_bounds__(256) zero_list_kernel(ZeroList z)
-{
-    float* p = z.p[blockIdx.x];
-    const int n = z.n[blockIdx.x];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = 0.f;
-}
-
 // SM count of the calling thread's current device, read on every launch (a
 // cheap attribute query), so a process driving parts of different sizes gets
 // each one's own persistent grid.
@@ -1306,11 +1294,10 @@ le_status decode_fused(int32_t P, const float* feat, const float* unc, const le_
         // the loss and the weight gradients the kernel adds into, zeroed by one launch
         const ZeroList zl{{loss, dg->W1, dg->b1, dg->W2, dg->b2, dg->W3, dg->b3, loss_l1},
                           {2, kH1 * kD, kH1, kH2 * kH1, kH2, a.ncb * kH2, a.ncb, 1}};
-        zero_list_kernel<<<img ? 8 : 7, 256, 0, s>>>(zl);
-        LE_LAUNCHED();
-        const size_t smem = train_smem(a.ncb);
-        le_status st = set_smem(dec_train_kernel, smem);
+        le_status st = zero_list(zl, img ? 8 : 7, s);
         if (st != LE_OK) return st;
+        const size_t smem = train_smem(a.ncb);
+        if ((st = set_smem(dec_train_kernel, smem)) != LE_OK) return st;
         const int grid = ntiles < sm_count() ? ntiles : sm_count();
         dec_train_kernel<<<grid, kTrainThreads, smem, s>>>(a);
         LE_LAUNCHED();

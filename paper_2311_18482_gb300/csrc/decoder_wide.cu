@@ -719,13 +719,9 @@ le_status wide_decode(int32_t P, const float* feat, const float* unc, const le_d
         LE_LAUNCHED();
         return LE_OK;
     }
-    LE_CUDA(cudaMemsetAsync(loss, 0, 2 * sizeof(float), s));
-    LE_CUDA(cudaMemsetAsync(dg->W1, 0, sizeof(float) * kW1 * 8, s));
-    LE_CUDA(cudaMemsetAsync(dg->b1, 0, sizeof(float) * kW1, s));
-    LE_CUDA(cudaMemsetAsync(dg->W2, 0, sizeof(float) * kW2 * kW1, s));
-    LE_CUDA(cudaMemsetAsync(dg->b2, 0, sizeof(float) * kW2, s));
-    LE_CUDA(cudaMemsetAsync(dg->W3, 0, sizeof(float) * ncb * kW2, s));
-    LE_CUDA(cudaMemsetAsync(dg->b3, 0, sizeof(float) * ncb, s));
+    const ZeroList zl{{loss, dg->W1, dg->b1, dg->W2, dg->b2, dg->W3, dg->b3},
+                      {2, kW1 * 8, kW1, kW2 * kW1, kW2, ncb * kW2, ncb}};
+    if ((st = zero_list(zl, 7, s)) != LE_OK) return st;
     LE_CUDA(cudaFuncSetAttribute(wide_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
     wide_kernel<true><<<grid, kThreads, kSmem, s>>>(a);
     LE_LAUNCHED();

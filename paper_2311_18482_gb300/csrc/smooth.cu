@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(kThreadsS, 1) smooth_kernel(SmoothArgs a)
     c.lanef = (uint32_t)(32 * (warp & 3)) << 16;
     // weights (BF16, [out][in]), biases (FP32), the ones operand
     sbuf_fill(SBuf{c.sm + kOW1, 16}, 128, a.W1, 3, kH, 3);
-    sbuf_fill(SBuf{c.sm + kOW2, kH}, 128, a.W2, kH, kH, kH);
-    sbuf_fill(SBuf{c.sm + kOW3, kH}, 128, a.W3, kH, kH, kH);
+    sbuf_fill_rows(SBuf{c.sm + kOW2, kH}, 128, a.W2);
+    sbuf_fill_rows(SBuf{c.sm + kOW3, kH}, 128, a.W3);
     sbuf_fill(SBuf{c.sm + kOW4, kH}, 16, a.W4, kH, kS, kH);
     float* bs = reinterpret_cast<float*>(c.sm + kOB);
     for (int i = threadIdx.x; i < 3 * kH + 16; i += blockDim.x)
@@ -452,10 +452,10 @@ extern "C" le_status le_smooth(int32_t n, const float* means, const float* feat,
     LE_CHECK_ARG(d_feat_stride >= 8, "d_feat_stride = %d < 8", d_feat_stride);
     LE_CHECK_ARG(n == 0 || aligned16(feat), "feat must be 16-byte aligned");
     cudaStream_t s = as_stream(stream);
-    LE_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
-    float* const gz[8] = {dmlp->W1, dmlp->b1, dmlp->W2, dmlp->b2, dmlp->W3, dmlp->b3, dmlp->W4, dmlp->b4};
-    const size_t gn[8] = {kH * 3, kH, kH * kH, kH, kH * kH, kH, kS * kH, kS};
-    for (int i = 0; i < 8; ++i) LE_CUDA(cudaMemsetAsync(gz[i], 0, gn[i] * sizeof(float), s));
+    const tc::ZeroList zl{{loss, dmlp->W1, dmlp->b1, dmlp->W2, dmlp->b2, dmlp->W3, dmlp->b3, dmlp->W4, dmlp->b4},
+                          {1, kH * 3, kH, kH * kH, kH, kH * kH, kH, kS * kH, kS}};
+    const le_status zs = tc::zero_list(zl, 9, s);
+    if (zs != LE_OK) return zs;
     if (n == 0) return LE_OK;
     int dev = 0, sms = 0;
     LE_CUDA(cudaGetDevice(&dev));
