@@ -143,7 +143,7 @@ le_status le_preprocess(const le_gaussians* g, const le_camera* cam, le_projecte
  * + 1) clipped to the rect, none if mm < dR^2 or mm < dL^2; the left-out
  * tiles hold no pixel where the renderer's alpha reaches 1/255, so images and
  * gradients equal those of whole-rect binning.  The K copies are never sorted:
- * the Gaussians are radix-sorted by depth, per-(tile, chunk-of-Gaussians)
+ * the Gaussians are sorted by depth, per-(tile, chunk-of-Gaussians)
  * copy counts come from per-row difference arrays of those spans, one
  * exclusive scan of the counts in tile-major order gives every chunk's offset
  * inside every tile's range, and each chunk writes its copies in depth order
@@ -395,7 +395,7 @@ le_status le_query(int32_t mode, int32_t P, const float* feat, const le_decoder*
  *   16-byte aligned; workspace: le_feature_map_workspace(n_cb, d) bytes.
  * One tcgen05 kernel: decode, softmax (stored in BF16, normalised in FP32 at
  * the output), F = p S with FP32 accumulation, BF16 out through TMA tensor
- * stores.  The workspace holds BF16 images of the codebook and of W3.
+ * stores.  The workspace holds a BF16 image of the codebook.
  * Errors: LE_ERR_INVALID_ARG; LE_ERR_UNSUPPORTED unless d is a multiple of
  * 64 and the decoder has the fused path's sizes. */
 le_status le_feature_map_workspace(int32_t n_cb, int32_t d, size_t* bytes);
