@@ -1178,9 +1178,10 @@ __global__ void codebook_chunks_kernel(const float* __restrict__ S, int ncb, int
 //   rows 0 - 15:     [text; negs] S_c^T (rows past Q + n_neg zero)
 //   rows 16 - ...:   G = S_c S_c^T
 // in blocks of 32 codes, each an [rows x 32] canonical buffer.  Bound by the latency
-// of its loads: 128 columns of both operands a step, read as 16-byte words (256 codes
-// against 2,073,600 pixels 730 -> 725 us, 64 codes against 72,261 37.2 -> 31.7 us; 32
-// columns a step and single words before).
+// of its loads: 128 columns of both operands a step, read as 16-byte words, the next
+// step's loads under this step's products (256 codes against 2,073,600 pixels 730 ->
+// 714 us, 64 codes against 72,261 37.2 -> 27.0 us; 32 columns a step, loaded as they
+// were needed, and single words before).
 __global__ void __launch_bounds__(256) query_prep_kernel(const float* __restrict__ S, int ncb, int dd, int d_clip,
                                                          const float* __restrict__ text, int Q,
                                                          const float* __restrict__ negs, int n_neg,
@@ -1191,20 +1192,30 @@ __global__ void __launch_bounds__(256) query_prep_kernel(const float* __restrict
     const int j0 = blockIdx.x * 16, i0 = ((int)blockIdx.y - 1) * 16;
     const bool gram = i0 >= 0;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc = 0.f;
+    constexpr int kN = 16 * kK / 256;                // words of each operand per thread and step
+    float acc = 0.f, xr[kN], yr[kN];
+    const auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < kN; ++q) {
+            const int l = threadIdx.x + 256 * q, r = l / kK, k = k0 + l % kK;
+            xr[q] = yr[q] = 0.f;
+            if (k < d_clip) {
+                if (gram) xr[q] = S[(size_t)(i0 + r) * dd + k];
+                else if (r < Q) xr[q] = text[(size_t)r * d_clip + k];
+                else if (r < Q + n_neg) xr[q] = negs[(size_t)(r - Q) * d_clip + k];
+                yr[q] = S[(size_t)(j0 + r) * dd + k];
+            }
+        }
+    };
+    load(0);
     for (int k0 = 0; k0 < d_clip; k0 += kK) {
 #pragma unroll
-        for (int l = threadIdx.x; l < 16 * kK; l += 256) {
-            const int r = l / kK, c = l % kK, k = k0 + c;
-            float xv = 0.f;
-            if (k < d_clip) {
-                if (gram) xv = S[(size_t)(i0 + r) * dd + k];
-                else if (r < Q) xv = text[(size_t)r * d_clip + k];
-                else if (r < Q + n_neg) xv = negs[(size_t)(r - Q) * d_clip + k];
-            }
-            xs[r][c] = xv;
-            ys[r][c] = k < d_clip ? S[(size_t)(j0 + r) * dd + k] : 0.f;
+        for (int q = 0; q < kN; ++q) {
+            const int l = threadIdx.x + 256 * q;
+            xs[l / kK][l % kK] = xr[q];
+            ys[l / kK][l % kK] = yr[q];
         }
+        load(k0 + kK);                               // past the end: zeros, no access
         __syncthreads();
 #pragma unroll 8
         for (int c = 0; c < kK; c += 4) {
