@@ -379,7 +379,8 @@ le_status le_decode_l1(int32_t mode, int32_t P, const float* feat, const float* 
  *     relevancy in one tcgen05 kernel using |F_clip|^2 = p^T (S_c S_c^T) p and
  *     phi.q = p.(S_c q) / |F_clip| (never forms F).
  * dec is required in both modes (its n_cb is the codebook size).  Q >= 1,
- * n_neg >= 1, Q + n_neg <= 16. */
+ * n_neg >= 1, Q + n_neg <= 16.  workspace: le_query_workspace bytes, 16-byte
+ * aligned (4-byte for the unfused mode). */
 le_status le_query_workspace(int32_t mode, int32_t P, int32_t n_cb, int32_t d_clip, size_t* bytes);
 le_status le_query(int32_t mode, int32_t P, const float* feat, const le_decoder* dec, const float* prob,
                    const float* codebook, int32_t d, int32_t d_clip, const float* text, int32_t Q,
@@ -520,7 +521,8 @@ le_status le_smooth(int32_t n, const float* means, const float* feat, const floa
  *   are carried for kept Gaussians and zero for clones and children.
  *   noise: [n,2,3] standard normal samples (the caller draws them).
  *   n_out: HOST pointer, the output count (also on LE_ERR_CAPACITY).
- *   workspace: le_densify_workspace(n) bytes.  Synchronizes `stream` once.
+ *   workspace: le_densify_workspace(n) bytes, 8-byte aligned.  Synchronizes
+ *   `stream` once.
  * Errors: LE_ERR_INVALID_ARG; LE_ERR_CAPACITY when the output exceeds n_cap. */
 typedef struct le_densify_config {
     float grad_thresh;       /* mean |dL/dmean2d| in pixels */
@@ -559,8 +561,8 @@ le_status le_rgb_l1(int64_t n, const float* img, const float* target, float* los
  * SSIM per channel with an 11 x 11 Gaussian window (sigma 1.5), zero padding
  * outside the image, C1 = 0.01^2, C2 = 0.03^2, mean over pixels and channels.
  *   img, target [3,H,W]; loss [3] out = (L, L1, SSIM); grad [3,H,W] out = dL/dimg;
- *   workspace: le_rgb_loss_workspace(W, H) bytes (the three per-pixel SSIM
- *   partial-derivative maps of every channel).
+ *   workspace: le_rgb_loss_workspace(W, H) bytes, 4-byte aligned (the three
+ *   per-pixel SSIM partial-derivative maps of every channel).
  * Errors: LE_ERR_INVALID_ARG (null pointers, bad size, lambda outside [0,1]). */
 le_status le_rgb_loss_workspace(int32_t W, int32_t H, size_t* bytes);
 le_status le_rgb_loss(int32_t W, int32_t H, const float* img, const float* target, float lambda_ssim, float* loss,

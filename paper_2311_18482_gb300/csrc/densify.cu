@@ -416,6 +416,7 @@ extern "C" le_status le_densify(const le_densify_config* cfg, const le_gaussians
     size_t need = 0;
     le_densify_workspace(n, &need);
     LE_CHECK_ARG(workspace_bytes >= need, "workspace has %zu bytes, needs %zu", workspace_bytes, need);
+    LE_CHECK_ARG((reinterpret_cast<uintptr_t>(workspace) & 7u) == 0, "workspace must be 8-byte aligned");
     const int nb = (n + kDB - 1) / kDB;
     unsigned char* w = static_cast<unsigned char*>(workspace);
     uint8_t* kind = w;

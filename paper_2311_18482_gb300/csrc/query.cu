@@ -93,6 +93,7 @@ extern "C" le_status le_query(int32_t mode, int32_t P, const float* feat, const 
         LE_CHECK_ARG(feat != nullptr, "fused query needs feat");
         need = query_fused_workspace(P, dec->n_cb, d_clip);
         LE_CHECK_ARG(workspace_bytes >= need && (need == 0 || workspace), "workspace too small");
+        LE_CHECK_ARG(aligned16(workspace), "workspace must be 16-byte aligned");
         return query_fused(P, feat, dec, codebook, d, d_clip, text, Q, negs, n_neg, relevancy, workspace,
                            workspace_bytes, s);
     }
@@ -100,6 +101,7 @@ extern "C" le_status le_query(int32_t mode, int32_t P, const float* feat, const 
     LE_CHECK_ARG(prob != nullptr, "unfused query needs prob");
     if ((st = le_query_workspace(mode, P, 1, d_clip, &need)) != LE_OK) return st;
     LE_CHECK_ARG(workspace && workspace_bytes >= need, "workspace too small: %zu < %zu", workspace_bytes, need);
+    LE_CHECK_ARG((reinterpret_cast<uintptr_t>(workspace) & 3u) == 0, "workspace must be 4-byte aligned");
     // n_cb is implied by the codebook pointer contract: prob is [n_cb, P], codebook [n_cb, d]
     const int n_cb = dec ? dec->n_cb : 0;
     LE_CHECK_ARG(n_cb > 0, "unfused query needs dec->n_cb for the codebook size");

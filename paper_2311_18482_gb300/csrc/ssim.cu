@@ -226,6 +226,7 @@ extern "C" le_status le_rgb_loss(int32_t W, int32_t H, const float* img, const f
     LE_CHECK_ARG(img && target && loss && grad && workspace, "null pointer");
     LE_CHECK_ARG(lambda_ssim >= 0.f && lambda_ssim <= 1.f, "lambda_ssim must be in [0, 1]");
     LE_CHECK_ARG(workspace_bytes >= ((size_t)9 * W * H + 64) * sizeof(float), "workspace too small");
+    LE_CHECK_ARG((reinterpret_cast<uintptr_t>(workspace) & 3u) == 0, "workspace must be 4-byte aligned");
     cudaStream_t s = as_stream(stream);
     float* maps = static_cast<float*>(workspace);
     float* acc = maps + (size_t)9 * W * H;

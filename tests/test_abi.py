@@ -76,3 +76,28 @@ def test_invalid_arguments_rejected_on_host(lib):
     assert lib.le_adam(C.c_int64(8), C.c_void_p(16), C.c_void_p(16), C.c_void_p(32), C.c_void_p(48), 0,
                        C.c_float(1e-3), C.c_float(0.9), C.c_float(0.999), C.c_float(1e-8), C.c_float(0),
                        C.c_float(1), None) == b.LE_ERR_INVALID_ARG
+
+
+def test_misaligned_workspaces_rejected_on_host(lib):
+    """A workspace that starts off the boundary its kernels' accesses need is refused before any launch."""
+    from paper_2311_18482_gb300 import binding as b
+    lib.le_last_error.restype = C.c_char_p
+    V, i, f, n = C.c_void_p, C.c_int32, C.c_float, C.c_size_t
+    p, big = V(256), n(1 << 30)
+
+    def refused(status):
+        assert status == b.LE_ERR_INVALID_ARG and b"aligned" in lib.le_last_error()
+
+    dec = b.LeDecoder()
+    dec.d_in, dec.h1, dec.h2, dec.n_cb = 8, 64, 128, 64
+    for k in ("W1", "b1", "W2", "b2", "W3", "b3"):
+        setattr(dec, k, 256)
+    for mode, at in ((b.FUSED_BF16, 264), (b.FUSED_BF16, 257), (b.UNFUSED_FP32, 258)):
+        refused(lib.le_query(i(mode), i(100), p, C.byref(dec), p, p, i(64), i(64), p, i(1), p, i(1), p, V(at), big,
+                             None))
+    refused(lib.le_rgb_loss(i(16), i(16), p, p, f(0.2), p, p, V(258), big, None))
+    g = b.LeGaussians(10, 0, *[256] * 7)
+    o = b.LeGaussianGrads(*[256] * 7)
+    cfg, out = b.LeDensifyConfig(0.1, 0.1, 1.0, 0.1, 0.0, 0.0), C.c_int64()
+    refused(lib.le_densify(C.byref(cfg), C.byref(g), C.byref(o), C.byref(o), p, p, None, p, C.c_int64(20), C.byref(o),
+                           C.byref(o), C.byref(o), C.byref(out), V(260), big, None))
