@@ -194,10 +194,18 @@ def reset_launch_count():
 
 
 # ---------------------------------------------------------------------------
+def _floats(a):
+    """A C array of any values that convert to float one by one: an array, a tensor, a list, an iterator."""
+    try:
+        v = [*map(float, a.tolist())]            # one conversion of an array for all its elements
+    except (AttributeError, TypeError):
+        v = [*map(float, a)]
+    return (C.c_float * len(v))(*v)
+
+
 def camera_struct(cam) -> LeCamera:
-    floats = lambda a: (C.c_float * len(a))(*map(float, a.tolist() if hasattr(a, "tolist") else a))
-    return LeCamera(floats(cam.view), floats(cam.campos), float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy),
-                    int(cam.W), int(cam.H), float(cam.near), floats(cam.bg))
+    return LeCamera(_floats(cam.view), _floats(cam.campos), float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy),
+                    int(cam.W), int(cam.H), float(cam.near), _floats(cam.bg))
 
 
 @dataclass

@@ -101,3 +101,25 @@ def test_misaligned_workspaces_rejected_on_host(lib):
     cfg, out = b.LeDensifyConfig(0.1, 0.1, 1.0, 0.1, 0.0, 0.0), C.c_int64()
     refused(lib.le_densify(C.byref(cfg), C.byref(g), C.byref(o), C.byref(o), p, p, None, p, C.c_int64(20), C.byref(o),
                            C.byref(o), C.byref(o), C.byref(out), V(260), big, None))
+
+
+def test_camera_takes_any_float_like_values():
+    """Lists, arrays, one-column tensors and iterators give the same camera; a wrong count is refused."""
+    import numpy as np
+    import torch
+    from types import SimpleNamespace
+    from paper_2311_18482_gb300 import binding as b
+    view, campos, bg = np.arange(12) / 7, np.array([1.5, -2, 3]), np.array([0.25, 0.5, 1])
+
+    def camera(f, view=view):
+        return bytes(b.camera_struct(SimpleNamespace(view=f(view), campos=f(campos), bg=f(bg), fx=1.0, fy=2, cx=3.5,
+                                                     cy=4, W=16, H=8, near=0.2)))
+
+    want = camera(lambda a: a)
+    for form in (list, iter, tuple, lambda a: a.astype(np.float32), lambda a: map(float, a), torch.tensor,
+                 lambda a: torch.tensor(a)[:, None], lambda a: [np.float32(v) for v in a],
+                 lambda a: (v for v in a.tolist())):
+        assert camera(form) == want
+    for n in (11, 13):
+        with pytest.raises((TypeError, ValueError)):
+            camera(list, view=np.ones(n))
