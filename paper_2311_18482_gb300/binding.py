@@ -238,8 +238,12 @@ class Gaussians:
                 self.opacity_raw.data_ptr(), self.sh.data_ptr(), self.feat.data_ptr(), self.unc.data_ptr())
 
     def empty_like(self) -> "Gaussians":
-        return Gaussians(*(torch.empty_like(getattr(self, k)) for k in
-                           ("means", "log_scales", "quats", "opacity_raw", "sh", "feat", "unc")), self.sh_degree)
+        """For gradients, which the calls write whole: rows of n Gaussians of sh_degree.  Where a tensor holds
+        more than those (its tail is not a parameter of the call), zeros."""
+        widths = (3, 3, 4, 1, 3 * (self.sh_degree + 1) ** 2, 8, 1)
+        like = lambda t, w: (torch.empty_like if t.numel() == self.n * w else torch.zeros_like)(t)
+        return Gaussians(*(like(getattr(self, k), w) for k, w in zip(
+            ("means", "log_scales", "quats", "opacity_raw", "sh", "feat", "unc"), widths)), self.sh_degree)
 
     def zeros_like(self) -> "Gaussians":
         return Gaussians(*(torch.zeros_like(getattr(self, k)) for k in

@@ -123,3 +123,18 @@ def test_camera_takes_any_float_like_values():
     for n in (11, 13):
         with pytest.raises((TypeError, ValueError)):
             camera(list, view=np.ones(n))
+
+
+def test_gradients_beyond_the_parameters_are_zero(monkeypatch):
+    """Gradient tensors come uninitialised where a backward writes every element; what a tensor holds past the
+    rows of n and sh_degree, which no call writes, starts as zeros."""
+    import torch
+    from paper_2311_18482_gb300 import binding as b
+    monkeypatch.setattr(torch, "empty_like", lambda t: torch.full_like(t, float("nan")))
+    n, nan = 5, lambda t: bool(torch.isnan(t).all())
+    make = lambda sh, feat: b.Gaussians(torch.ones(n, 3), torch.ones(n, 3), torch.ones(n, 4), torch.ones(n), sh, feat,
+                                        torch.ones(n), 1).empty_like()
+    exact = make(torch.ones(n, 4, 3), torch.ones(n, 8))
+    assert all(nan(getattr(exact, k)) for k in ("means", "log_scales", "quats", "opacity_raw", "sh", "feat", "unc"))
+    wide = make(torch.ones(n, 16, 3), torch.ones(n, 9))
+    assert not wide.sh.any() and not wide.feat.any() and wide.sh.shape == (n, 16, 3) and nan(wide.means)
