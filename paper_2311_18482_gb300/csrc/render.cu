@@ -430,7 +430,9 @@ __global__ void __launch_bounds__(kBlock / PPT) render_bwd_kernel(
                             acc[k] = __ffma2_rn(wb, dC[2 * p + 1][k], acc[k]);
                         }
                         const float2 fdc = make_float2(__fadd_rn(ea.x, ea.y), __fadd_rn(eb.x, eb.y));
-                        const float2 diff = __fadd2_rn(fdc, make_float2(-S[p].x, -S[p].y));
+                        float2 diff = __fadd2_rn(fdc, make_float2(-S[p].x, -S[p].y));
+                        // a non-finite channel stays with the pixels that blend it (0 times it is not 0)
+                        if (U > 1) diff = sel2(cx, cy, diff);
                         const float2 dal = __ffma2_rn(T[p], diff, __fmul2_rn(__fmul2_rn(Tf[p], inv), nbg[p]));
                         S[p] = __ffma2_rn(am, diff, S[p]);
                         // alpha below the 0.99 clamp: dalpha/dpower = alpha, dalpha/do = G

@@ -123,6 +123,45 @@ def test_backward_few_and_many_tiles(leg, orc, W, H):
     assert rel_err(to_np(grads.unc), g2["unc"]) < 1e-4
 
 
+@pytest.mark.parametrize("W,H", [(16, 16), (512, 320)])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_backward_keeps_non_finite_channels_to_their_pixels(leg, W, H, bad):
+    """Two Gaussians in one tile, no pixel blending both: the gradients of the nearer one are bit for bit the
+    same whether or not a channel of the other is finite, in both layouts of the backward (1 and 640 tiles)."""
+    cam = synth.look_at_camera((0.0, 0.0, -3.0), (0.0, 0.0, 0.0), (0.0, 1.0, 0.0), W, H, 60.0)
+    cam.fx, cam.fy, cam.cx, cam.cy = 100.0, 100.0, 7.5, 7.5
+    z = np.array([3.0, 4.0])                        # camera depths; pixels (12, 6) and (3, 6)
+    px = np.array([12.0, 3.0])
+    means = np.stack([(px - cam.cx) * z / cam.fx, (6.0 - cam.cy) * z / cam.fy, z], 1)
+    R = np.asarray(cam.view, np.float64).reshape(3, 4)
+    means = (means - R[:, 3]) @ R[:, :3]            # back into the world
+    quats = np.tile(np.array([1.0, 0, 0, 0]), (2, 1))
+    rng = np.random.default_rng(3)
+    up = [_t(a) for a in upstream(rng, H, W)]
+    fixed = (_t(means), _t(np.full((2, 3), -6.0)), _t(quats), _t(np.full(2, 2.0)), _t(rng.uniform(-1, 1, (2, 1, 3))))
+    feat, unc = rng.standard_normal((2, 8)), _t(rng.uniform(0, 1, 2))
+
+    def grads():
+        g = leg.Gaussians(*fixed, _t(feat), unc, 0)
+        proj = leg.le_preprocess(g, cam)
+        ids, ranges, K, _ = leg.le_bin_sort(cam, proj)
+        img = leg.le_render_fwd(cam, proj, ids, ranges)
+        out, grad2d = leg.le_render_bwd(cam, g, proj, ids, ranges, img, *up)
+        torch.cuda.synchronize()
+        assert K == 2 and np.abs(to_np(proj.splat[:, 0]) - px).max() < 1e-2
+        assert int(img.n_contrib[6, 12]) == 1 and int(img.n_contrib[6, 3]) == 2
+        return {k: to_np(getattr(out, k))[0] for k in ("means", "log_scales", "quats", "opacity_raw", "sh", "feat",
+                                                       "unc")}, to_np(grad2d)[0]
+
+    want, want2d = grads()
+    assert np.abs(want2d[:18]).min() > 0
+    feat[1, 5] = bad
+    got, got2d = grads()
+    assert np.array_equal(got2d[:18], want2d[:18])
+    for k, v in want.items():
+        assert np.array_equal(got[k], v), k
+
+
 def test_autograd_function(leg, orc):
     c = synth.config("c1", n=800, W=64, H=64)
     sc, cam = c["scene"], c["camera"]
