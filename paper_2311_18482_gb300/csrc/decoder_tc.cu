@@ -842,6 +842,7 @@ struct ExportBars {                          // of one tile slot
     uint64_t full[kXSlots], empty[kXSlots];  // codebook slots
     uint64_t acc_full, acc_free;             // a chunk's accumulator
     uint64_t e_ready;                        // the tile's e is in tensor memory
+    uint64_t begun;                          // e_ready of the slot's first tile: completes once
     uint64_t front, fin;
 };
 
@@ -875,6 +876,7 @@ __device__ __forceinline__ void decode_contract(const CUtensorMap* tmap_out, con
         mbar_init(&b->acc_full, 1);
         mbar_init(&b->acc_free, 8);
         mbar_init(&b->e_ready, 1);
+        mbar_init(&b->begun, 1);
         mbar_init(&b->front, 1);
         mbar_init(&b->fin, 1);
     }
@@ -982,8 +984,9 @@ __device__ __forceinline__ void decode_contract(const CUtensorMap* tmap_out, con
         const int rest0 = f.half ? hu + held : 0, rest1 = f.half ? nu : hu;
         float xf[8];                                // this tile's R_s (half 0), in L2 a tile ahead
         if (f.half == 0) load_feat(a, first * 128 + row, first < ntiles && first * 128 + row < a.P, xf);
-        // out of phase with the first slot
-        if (t == 1 && first < ntiles) ok = !bar_any(f.bar_id, 256, !mbar_wait(&bars->e_ready, 0));
+        // out of phase with the first slot (a barrier of its own: e_ready's parity comes round again with every
+        // second tile, so a thread that looked late would wait for a tile that may not come)
+        if (t == 1 && first < ntiles) ok = !bar_any(f.bar_id, 256, !mbar_wait(&bars->begun, 0));
         uint32_t c = 0;
         for (int tile = first; tile < ntiles && ok; tile += stride) {
             const bool valid = tile * 128 + row < a.P;
@@ -1041,7 +1044,10 @@ __device__ __forceinline__ void decode_contract(const CUtensorMap* tmap_out, con
             fence_before();
             wg_sync(f);
             fence_after();
-            if (lead && f.half == 0) mbar_arrive(&bar->e_ready);
+            if (lead && f.half == 0) {
+                mbar_arrive(&bar->e_ready);
+                if (tile == first) mbar_arrive(&bar->begun);
+            }
             const float inv = !QUERY && valid ? 1.0f / (sums[2 * t * 128 + row] + sums[(2 * t + 1) * 128 + row]) : 0.f;
             float pj[16], quad = 0.f;               // query: the projections (half 0), e^T G e over this half's columns
             for (int j = 0; j < nch; ++j, ++c) {
