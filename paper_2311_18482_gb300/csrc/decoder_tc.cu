@@ -1238,14 +1238,15 @@ __global__ void __launch_bounds__(256) query_prep_kernel(const float* __restrict
     *reinterpret_cast<__nv_bfloat16*>(blk + sbuf_off(r - j * kXDims, c % kXCodes, kXCodes)) = __float2bfloat16_rn(acc);
 }
 
-// Self-test of the bounded-wait path: waits on an mbarrier that nothing ever
-// arrives at, gives up after the usual limit and records the timeout.
+// Self-test of the bounded-wait path: one thread, not the one that records,
+// waits on an mbarrier that nothing ever arrives at, gives up after the usual
+// limit, and the block puts the timeout on record.
 __global__ void selftest_wait_kernel()
 {
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
-    if (threadIdx.x == 0 && !mbar_wait(&bar, 0u)) atomicExch(&g_tc_error, 1);
+    (void)cta_failed(threadIdx.x != 5 || mbar_wait(&bar, 0u), &g_tc_error);
 }
 
 // SM count of the calling thread's current device, read on every launch (a

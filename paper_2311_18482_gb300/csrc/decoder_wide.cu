@@ -578,11 +578,10 @@ __global__ void __launch_bounds__(kRows, 1) wide_wgrad_kernel(WgradArgs a)
             }
         }
         // the last half-tile's MMAs
-        if (ok && nq > 0 && !mbar_wait(empty + (nq - 1) % kWStages, (uint32_t)((nq - 1) / kWStages) & 1u))
-            ok = false;
-        if (!ok && tid == 0) atomicExch(&g_wide_error, 1);
+        if (ok && nq > 0)
+            ok = warp_agree(mbar_wait(empty + (nq - 1) % kWStages, (uint32_t)((nq - 1) / kWStages) & 1u));
     }
-    const bool bad = bar_any(0, kRows, !ok);
+    const bool bad = cta_failed(ok, &g_wide_error);
     fence_after();
     if (!bad && n > 0) {
         const uint32_t tl = tbase + ((uint32_t)(32 * (tid >> 5)) << 16);

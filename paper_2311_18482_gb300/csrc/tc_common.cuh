@@ -143,6 +143,15 @@ __device__ __forceinline__ uint32_t warp_uniform(uint32_t x) { return __shfl_syn
 // leaves part of them at the next elect_one().
 __device__ __forceinline__ bool warp_agree(bool ok) { return __all_sync(0xffffffffu, ok); }
 
+// A barrier of the whole CTA that joins its threads' outcomes: true for all if any of them gave up, which is
+// then on record (each thread has a clock of its own, so any one of them may be the only one).
+__device__ __forceinline__ bool cta_failed(bool ok, int* error)
+{
+    const bool bad = __syncthreads_or(!ok);
+    if (bad && threadIdx.x == 0) atomicExch(error, 1);
+    return bad;
+}
+
 // D[tmem] (+)= A * B, issued by one thread.
 __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
 {
