@@ -123,6 +123,12 @@ def test_backward_few_and_many_tiles(leg, orc, W, H):
     assert rel_err(to_np(grads.unc), g2["unc"]) < 1e-4
 
 
+@pytest.mark.parametrize("W,H", [(384, 304), (400, 304)])
+def test_backward_layouts_at_their_line(leg, orc, W, H):
+    """The last image size of the two-pixel layout (456 tiles) and the first of the four-pixel one."""
+    test_backward_few_and_many_tiles(leg, orc, W, H)
+
+
 @pytest.mark.parametrize("W,H", [(16, 16), (512, 320)])
 @pytest.mark.parametrize("bad", [float("inf"), float("nan")])
 def test_backward_keeps_non_finite_channels_to_their_pixels(leg, W, H, bad):
