@@ -106,6 +106,14 @@ def test_densify_rows_of_every_width(leg, orc, n, degree, offset):
             assert np.array_equal(getattr(g, k).cpu().numpy()[:exact], ref[k][:exact].astype(np.float32)), k
 
 
+@pytest.mark.parametrize("degree,offset", [(3, 0), (2, 0), (0, 1)])
+@pytest.mark.parametrize("n", [88576, 88877])
+def test_densify_on_both_grids(leg, orc, n, degree, offset):
+    """The last count whose fields have blocks of their own (173 blocks of 512 Gaussians each) and one whose
+    blocks copy all seven, with 16-byte and scalar rows: the copies are exact."""
+    test_densify_rows_of_every_width(leg, orc, n, degree, offset)
+
+
 def test_densify_capacity(leg):
     P, acc, cnt = _densify_inputs(3000, 83)
     noise = torch.zeros((3000, 2, 3), device="cuda")
