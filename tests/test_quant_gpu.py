@@ -64,6 +64,14 @@ def test_quantize_other_split(leg, orc):
     _check(orc, F, S, idx, r, p, loss, d_clip=128)
 
 
+def test_quantize_several_tiles_per_cta(leg, orc):
+    """Three and four tiles for every CTA (469 tiles, the last one ragged): accumulator, norm and exchange slots
+    are reused from the third on.  256-dim features keep the oracle quick."""
+    F, S = synth.quant_inputs(9, 60001, 128, d_clip=128, d_dino=128)
+    idx, r, p, loss = _run(leg, F, S, d_clip=128)
+    _check(orc, F, S, idx, r, p, loss, d_clip=128)
+
+
 def test_quantize_features_equal_codes(leg, orc):
     """Features that are the (BF16-rounded) codes themselves: m_i = the code, L_cos = 0 up to FP32 rounding."""
     rng = np.random.default_rng(8)
@@ -135,6 +143,27 @@ def test_quantize_grad_parity(leg, orc, K, N):
     mx = np.abs(Gr - Go).max() / np.abs(Go).max()
     print(f"K={K} N={N}: rel Frobenius {fro:.2e}, max {mx:.2e}")
     assert fro <= 1e-2 and mx <= 2e-2
+
+
+@pytest.mark.parametrize("K,N,d_clip,d_dino", [(3001, 16, 512, 384), (3001, 48, 512, 384), (3001, 80, 512, 384),
+                                               (3001, 112, 512, 384), (60001, 128, 128, 128)])
+def test_quantize_grad_parts_and_tiles(leg, orc, K, N, d_clip, d_dino):
+    """The epilogue's four column parts where some are empty or shorter (16, 48, 80, 112 codes), and an odd K of
+    three and four tiles per CTA: the bars of test_quantize_grad_parity."""
+    rng = np.random.default_rng(70 + N)
+    cen = np.concatenate([synth.unit_rows(rng, N, d_clip), synth.unit_rows(rng, N, d_dino)], axis=1).astype(np.float32)
+    d = d_clip + d_dino
+    F = synth._bf16_bits(cen[rng.integers(0, N, K)] +
+                         rng.standard_normal((K, d)).astype(np.float32) * np.float32(0.5 / np.sqrt(d)))
+    Ft, St = torch.from_numpy(F.view(np.int16)).cuda(), torch.from_numpy(cen).cuda()
+    idx, r, _, _ = leg.le_quantize(Ft, St, d_clip=d_clip)
+    G = leg.le_quantize_grad(Ft, St, r, d_clip=d_clip)
+    torch.cuda.synchronize()
+    o = orc.quantize(F, cen, d_clip=d_clip, want_grad=True)
+    assert np.array_equal(idx.cpu().numpy(), o["m"])
+    Gr, Go = G.cpu().numpy().astype(np.float64), o["grad_S"]
+    assert np.linalg.norm(Gr - Go) <= 1e-2 * np.linalg.norm(Go)
+    assert np.abs(Gr - Go).max() <= 2e-2 * np.abs(Go).max()
 
 
 def test_quantize_grad_descends(leg, orc):

@@ -104,6 +104,12 @@ def test_smooth_vs_bf16_emulation_and_oracle(leg, orc, n):
         assert _rel(got["d" + k], ref["d" + k]) <= bars[k], k
 
 
+def test_smooth_several_tiles_per_cta(leg, orc):
+    """Three and four tiles for every CTA (469 tiles, the last one ragged): a tile's buffers and barriers are
+    reused two tiles later."""
+    test_smooth_vs_bf16_emulation_and_oracle(leg, orc, 60001)
+
+
 # (offset, stride) in floats: grad2d's feature slots (8-byte aligned rows), an odd offset (4-byte
 # aligned rows), a 16-byte aligned strided layout
 @pytest.mark.parametrize("off,stride", [(10, 20), (9, 20), (12, 24)])
