@@ -187,8 +187,9 @@ constexpr int kSortWarps = kSortThreads / 32;
 // long as one tile does while every tile has an SM of its own.  le_bin_sort with
 // tiles of 1,024 / 2,048 / 4,096 elements: 100,000 Gaussians 138 / 148 / 176 us,
 // 400,000 152 / 158 / 180, 600,000 203 / 193 / 202, 1M 269 / 255 / 266, 3M 638 /
-// 583 / 591.  The largest tiles remain for counts whose digit table would not fit
-// where the smaller ones' lies (from 134M).
+// 583 / 591.  The largest tiles, whose digit counts have a segment of their own,
+// remain above 2^26 Gaussians: the smaller ones' counts lie in the copy-count table
+// (64 MB from 524,288 Gaussians on), half of which they take at that size.
 inline int sort_items(int n) { return n <= 450000 ? 2 : (n <= 1 << 26 ? 4 : kSortItems); }
 
 __device__ __forceinline__ uint32_t digit_of(uint64_t e, int shift) { return (uint32_t)(e >> shift) & 255u; }
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64
     const int base = blockIdx.x * kTileElems;
     const int cnt = min(kTileElems, n - base);
 
-    // each warp owns the contiguous sub-range [w * 256, (w + 1) * 256) of the tile
+    // each warp owns a contiguous sub-range of 32 ITEMS elements of the tile
     const uint32_t lt = (1u << lane) - 1u;
     uint64_t e[ITEMS];
     uint32_t dg[ITEMS];

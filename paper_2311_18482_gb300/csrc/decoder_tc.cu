@@ -8,7 +8,8 @@
 // memory) and the softmax at the end.  Four kernels share that front end:
 //
 //   dec_fwd_kernel    inference (supp. Sec. "Inference"): argmax and/or
-//                     M_infer = softmax(logits), two tiles in flight per CTA.
+//                     M_infer = softmax(logits), four tiles in flight per CTA
+//                     (two above 128 codes).
 //   dec_train_kernel  training step (Eqs. 9-12): uncertainty-weighted CE,
 //                     dL/dR_u, and the whole backward on the tensor cores,
 //                     warp-specialised with two tiles in flight (one MMA
@@ -65,10 +66,9 @@ struct DecArgs {
     float inv_l1;
 };
 
-// Per-warpgroup state of the shared MLP front end.  With nhalf = 2 or 4,
-// that many warpgroups serve the same 128 TMEM lanes (rows) and split every
-// epilogue by columns; `xch` is their shared-memory exchange for row-wide
-// statistics ([nhalf][128] float4).
+// Per-warpgroup state of the shared MLP front end.  With nhalf = 2, two
+// warpgroups serve the same 128 TMEM lanes (rows) and split every epilogue by
+// columns; `xch` is their shared-memory exchange for row-wide statistics.
 struct Front {
     SBuf W1s, W2s, W3s, X1, H1, H2;
     const float *b1s, *b2s, *b3s;
@@ -80,7 +80,7 @@ struct Front {
     int bar_id, nthreads;
     bool issuer;       // the warp that issues this group's MMAs (warp-uniform)
     int half, nhalf;
-    float4* xch;       // [nhalf][128] (nhalf > 1 only)
+    float4* xch;       // [2][128] (nhalf = 2 only)
 };
 
 // Columns [c0, c1) of an N-column epilogue handled by this thread's half (units of 16).
@@ -93,8 +93,7 @@ __device__ __forceinline__ void my_cols(const Front& f, int N, int& c0, int& c1)
 
 __device__ __forceinline__ void wg_sync(const Front& f)
 {
-    if (f.nthreads == (int)blockDim.x) __syncthreads();
-    else asm volatile("bar.sync %0, %1;" ::"r"(f.bar_id), "r"(f.nthreads) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(f.bar_id), "r"(f.nthreads) : "memory");
 }
 
 // Wait for this warpgroup's MMA barrier; false (for every thread) if any thread timed out.
@@ -263,7 +262,7 @@ __global__ void __launch_bounds__(128 * NWG, 1) dec_fwd_kernel(DecArgs a)
     f.tid = threadIdx.x & 127;
     f.bar_id = 1 + wg;
     f.issuer = (warp & 3) == 0;
-    f.nthreads = NWG == 1 ? (int)blockDim.x : 128;
+    f.nthreads = 128;
     f.half = 0;
     f.nhalf = 1;
     f.xch = nullptr;
@@ -827,9 +826,9 @@ __global__ void __launch_bounds__(kTrainThreads, 1) dec_train_kernel(DecArgs a)
 // 0.812 ms, the same with e in shared memory 0.886 ms, one tile at a time in rounds
 // of two 64-dim chunks 1.255 ms.  Per tile, 45,000 cycles: 17,000 in the front,
 // 13,000 waiting for the codebook (the latency of four slots), 13,000 of MMAs.
-// A query of 2,073,600 pixels against 256 codes takes 0.730 ms, of 72,261 against
-// 64 codes 37 us (0.863 ms and 43 us with one tile at a time, four warpgroups on it
-// and G partly resident in shared memory).
+// A query of 2,073,600 pixels against 256 codes takes 0.714 ms, of 72,261 against
+// 64 codes 27 us (0.863 ms and 43 us with one tile at a time, four warpgroups on it
+// and G partly resident in shared memory, and the operand's preparation as it was).
 constexpr int kXSlots = 4, kXCodes = 32, kXDims = 128;
 constexpr uint32_t kXSlotBytes = sbuf_bytes(kXCodes, kXDims), kXBox = sbuf_bytes(128, 32);
 // A tile's region: X1 and H1, then H2 over them; in the back phase two staging boxes per warpgroup.
@@ -1163,7 +1162,7 @@ __global__ void __launch_bounds__(kXThreads, 1) query_fused_kernel(DecArgs a) { 
 
 // The export's codebook S [ncb x dd] (fp32) as a chunked canonical BF16 image:
 // chunk j holds dims [128 j, 128 j + 128) (64 in the last chunk of an odd multiple
-// of 64) of every code, as an [ncb x 128] canonical buffer, whose blocks of 64
+// of 64) of every code, as an [ncb x 128] canonical buffer, whose blocks of 32
 // codes are contiguous.
 __global__ void codebook_chunks_kernel(const float* __restrict__ S, int ncb, int dd, unsigned char* __restrict__ img)
 {

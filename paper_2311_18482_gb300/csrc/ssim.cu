@@ -12,8 +12,8 @@
 // ssim_bwd_kernel: the same two-pass blur of A, B, C; the gradient
 //   dL/dx = ((1 - lambda) sign(x - y) - lambda (G*A + 2 x G*B + y G*C)) / (3 P).
 // The two passes are bound by shared-memory reads, so a thread forms four
-// neighbouring outputs from 14 taps it reads once: 35 reads a pixel against 90
-// with one output per thread and 16 x 16 tiles, whose halo is also 2.6 times the
+// neighbouring outputs from 14 taps it reads once: the forward reads 28 words a pixel
+// against 91 with one output per thread and 16 x 16 tiles, whose halo is also 2.6 times the
 // tile instead of 1.7.  Loss and gradient of a 640 x 480 image: 39 us (58 us), of
 // 1296 x 840: 107 us (172 us).
 #include "common.cuh"

@@ -231,12 +231,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r)
 
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Store one FP32 value to a column of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_st1(uint32_t taddr, float v)
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(__float_as_uint(v)) : "memory");
-}
-
 // Single arrival on an mbarrier (release semantics at CTA scope).
 __device__ __forceinline__ void mbar_arrive(uint64_t* m)
 {
@@ -267,18 +261,6 @@ __device__ __forceinline__ void sbuf_store8(const SBuf& b, int r, int c0, const 
     *reinterpret_cast<uint4*>(b.p + sbuf_off(r, c0, b.C)) = *reinterpret_cast<uint4*>(h);
 }
 
-__device__ __forceinline__ void sbuf_load8(const SBuf& b, int r, int c0, float* v)
-{
-    const uint4 u = *reinterpret_cast<const uint4*>(b.p + sbuf_off(r, c0, b.C));
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float2 f = __bfloat1622float2(h[j]);
-        v[2 * j] = f.x;
-        v[2 * j + 1] = f.y;
-    }
-}
-
 // Descriptor of the (128-row or N-row) K-major block whose first row is row0,
 // K columns starting at k0 (both multiples of 8).
 __device__ __forceinline__ uint64_t kdesc(const SBuf& b, int row0, int k0)
@@ -286,14 +268,8 @@ __device__ __forceinline__ uint64_t kdesc(const SBuf& b, int row0, int k0)
     return make_desc(smem_u32(b.p) + sbuf_off(row0, k0, b.C), 128u, (uint32_t)(b.C >> 3) * 128u);
 }
 
-// Descriptor of the MN-major block: rows are K (starting at k0), columns are M/N
-// (starting at mn0).
-__device__ __forceinline__ uint64_t mndesc(const SBuf& b, int k0, int mn0)
-{
-    return make_desc(smem_u32(b.p) + sbuf_off(k0, mn0, b.C), (uint32_t)(b.C >> 3) * 128u, 128u);
-}
-
-// The same for a buffer given by its shared-memory address and column count.
+// The same for a buffer given by its shared-memory address and column count, and
+// the MN-major block: rows are K (starting at k0), columns are M/N (starting at mn0).
 __device__ __forceinline__ uint64_t kdesc_at(uint32_t base, int C, int row0, int k0)
 {
     return make_desc(base + sbuf_off(row0, k0, C), 128u, (uint32_t)(C >> 3) * 128u);
