@@ -532,7 +532,7 @@ namespace {
 // Up to three tiles per SM, a tile's serial walk sets the time: two pixels per
 // thread, two records at a time.  The line is where no measured scene loses: 21
 // scenes (300 to 1M Gaussians, opaque to nearly transparent, lists of 1 to 18,000)
-// in 19 image shapes of 304 to 475 tiles take 1.02 to 1.53 times as long with four
+// in 19 image shapes of 304 to 475 tiles take 1.01 to 1.53 times as long with four
 // pixels and one record, smaller images 1.15 to 1.66 times (64 tiles, 2,000
 // Gaussians 94 against 64 us; 256 tiles, 1M Gaussians 319 against 241).  From 494
 // tiles on it depends on the scene and the shape (608 tiles: 0.86 to 1.3 times).
